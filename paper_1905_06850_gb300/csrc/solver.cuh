@@ -886,7 +886,8 @@ __device__ __forceinline__ void op_apply(const StencilDesc &st, const CsrDesc &c
 template <typename T>
 struct Coef {
     int mode;                 // 0: fill (i < l), 1: recurrences (i >= l)
-    int k6;                   // 0: none, 1: phat_0 = v_0, 2: x and phat update (phat_m = eta_m p_m)
+    int k6;                   // 0: none, 1: phat_0 = v_0, 2: steps m - 1 and m of x and phat
+                              // (phat_m = eta_m p_m), 3: step m left to the next sweep, 4: step m
     int end;                  // -1: continue, else SegEnd
     int fmode;                // final sweep: 0 x += f1 phat; 1 lucky (m >= 1); 2 lucky (m = 0)
     int prev0;                // z^(0)_{m-1} exists
@@ -962,6 +963,7 @@ struct Smem {
     double bnorm[2];
     double raw2[kMaxDots];           // the scalar warp's copy of a reduced dot column
     Coef<T> cfb[2];                  // coefficients of iterations i (i & 1) and i + 1
+    T zxr[2], ppr[2];                // K6 in pairs: zx and pp of step m in slot (m >> 1) & 1, m odd
     long long stg_e0;                // CSR staging: global position of the unit's first staged entry
     int stg_on;                      // CSR staging: this unit's entries are in shared memory
     int ok;
@@ -1300,7 +1302,18 @@ __device__ __forceinline__ void step_vectors(Coef<T> &cf, const SolveArgs<T> &a,
 template <typename T, int L>
 constexpr bool kScaledBases = (sizeof(T) == 8 && L <= 5);
 
-template <typename T, int L, bool SC>
+// K6 in pairs: x and phat take steps m - 1 and m (m = i - l) together in the
+// sweeps of even m -- the first step's W_{m-1} = z^(0)_{m-1} is an operand of
+// K4 there -- so they pass through memory every second iteration: 3 l + 5
+// instead of 3 l + 7 vector passes, the same operations on every row (3D 256^3
+// FP32 p(1)-CG 59.5 -> 55.1 ms, the batch of 4096 2D systems 51.2 -> 47.5 ms,
+// same bits).  Not where vector traffic is not the bound: the FP64 p(1)-CG
+// sweep with scaled bases (FP64 units; 122.7 -> 123.8 ms in pairs) and CSR
+// (matrix traffic; short solves lose by the longer loop).
+template <typename T, int L, int OP, bool SC>
+constexpr bool kPairK6 = !op_is_csr(OP) && !(SC && L == 1 && sizeof(T) == 8);
+
+template <typename T, int L, bool SC, bool PAIR>
 __device__ __forceinline__ void scalar_step_body(Smem<T> &s, Coef<T> &cf, const double *raw,
                                                  const SolveArgs<T> &a, int i, double rn,
                                                  double tau, long long budget, T kc, T kn)
@@ -1326,6 +1339,7 @@ __device__ __forceinline__ void scalar_step_body(Smem<T> &s, Coef<T> &cf, const 
         }
         return;
     }
+    cf.f1 = T(0);
     const int c = i - L + 1;
     double *col = s.G[c % (L + 1)];
     // scales of this step: s_i, s_{i-1}, t_m = t^(0)_m, t_{m-1} (with
@@ -1494,10 +1508,14 @@ __device__ __forceinline__ void scalar_step_body(Smem<T> &s, Coef<T> &cf, const 
         cf.k6 = 1;
     } else {
         const double iep = s.ieta[(m - 1) & 1];
-        cf.k6 = 2;
+        cf.k6 = !PAIR ? 4 : (m & 1) ? 3 : 2;
         // scaled bases: P_m = phat_m / t_m = W_m - (delta_{m-1}/eta_{m-1})(t_{m-1}/t_m) P_{m-1}
         cf.zx = (T)(s.zeta[(m - 1) & 1] * iep * t_mm1);
         cf.pp = (T)(-dm1 * iep * (t_mm1 * it_m));
+        if (PAIR && (m & 1)) {
+            s.zxr[(m >> 1) & 1] = cf.zx;
+            s.ppr[(m >> 1) & 1] = cf.pp;
+        }
         s.eta[m & 1] = em;
         s.ieta[m & 1] = iem;
         s.zeta[m & 1] = zm;
@@ -1517,12 +1535,12 @@ __device__ __forceinline__ void scalar_step_body(Smem<T> &s, Coef<T> &cf, const 
     }
 }
 
-template <typename T, int L, bool SC>
+template <typename T, int L, bool SC, bool PAIR>
 __device__ __noinline__ void scalar_step_call(Smem<T> &s, Coef<T> &cf, const double *raw,
                                               const SolveArgs<T> &a, int i, double rn, double tau,
                                               long long budget, T kc, T kn)
 {
-    scalar_step_body<T, L, SC>(s, cf, raw, a, i, rn, tau, budget, kc, kn);
+    scalar_step_body<T, L, SC, PAIR>(s, cf, raw, a, i, rn, tau, budget, kc, kn);
 }
 
 // The scalar step inline, except in the FP32 whole-grid kernels: there the
@@ -1530,13 +1548,13 @@ __device__ __noinline__ void scalar_step_call(Smem<T> &s, Coef<T> &cf, const dou
 // changes its register allocation enough to cost ~15% at 256^3 (measured);
 // the out-of-line call costs ~0.3 us per iteration, which the FP64 and
 // one-CTA paths (latency-bound on small systems) keep.
-template <typename T, int L, bool OOL, bool SC>
+template <typename T, int L, bool OOL, bool SC, bool PAIR>
 __device__ __forceinline__ void scalar_step(Smem<T> &s, Coef<T> &cf, const double *raw,
                                             const SolveArgs<T> &a, int i, double rn, double tau,
                                             long long budget, T kc, T kn)
 {
-    if constexpr (OOL) scalar_step_call<T, L, SC>(s, cf, raw, a, i, rn, tau, budget, kc, kn);
-    else scalar_step_body<T, L, SC>(s, cf, raw, a, i, rn, tau, budget, kc, kn);
+    if constexpr (OOL) scalar_step_call<T, L, SC, PAIR>(s, cf, raw, a, i, rn, tau, budget, kc, kn);
+    else scalar_step_body<T, L, SC, PAIR>(s, cf, raw, a, i, rn, tau, budget, kc, kn);
 }
 
 // Per-thread accumulator of one dot product over the units a thread sweeps.
@@ -1675,6 +1693,7 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
     // FP64 p(1)-CG keeps its bases scaled (see scalar_step_body): two FP64
     // multiplies per row fewer in the FP64-bound sweep
     constexpr bool kScaled = SC && kScaledBases<T, L>;
+    constexpr bool kPair = kPairK6<T, L, OP, SC>;
     // CSR on the whole grid: each sweep unit's entries are bulk-copied into
     // shared memory (one contiguous range per unit) before its rows are read
     constexpr bool kStage = op_is_csr(OP) && std::is_same<Grp, GridGroup<T>>::value && RPT == 1;
@@ -1813,21 +1832,34 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
         // l iterations later) with the local work, on one GPU.
         const bool la = (L >= 2) && a.lookahead;
         const int nsw = la ? kBlock - 32 : kBlock;   // threads that sweep
-        if (tid == 0) scalar_step<T, L, kOolScalar, SC>(s, s.cfb[0], s.raw, a, 0, rn, tau, budget, kc, kn);
+        if (tid == 0) scalar_step<T, L, kOolScalar, SC, kPair>(s, s.cfb[0], s.raw, a, 0, rn, tau, budget, kc, kn);
         __syncthreads();
         for (long long i = 0;; ++i) {
             const Coef<T> &cf = s.cfb[i & 1];
+            // K6 in pairs: the first step's zx and pp (of step m - 1 = i - l - 1)
+            const int k6s = (int)((i + 3 - L) >> 1) & 1;
             if (cf.end >= 0) {
-                // ---- final vector update of the segment
-                if (cf.end != kSegNonfinite) {
+                // ---- final vector update of the segment (a segment that ends on
+                // a non-finite scalar takes the outstanding step alone)
+                const bool pend = kPair && i >= L + 2 && ((i - L) & 1) == 0;   // step m - 1 is outstanding
+                if (cf.end != kSegNonfinite || (!kF32 && pend)) {
                     for (int64_t u = grp.unit0(); u < nunits; u += grp.ustep()) {
                         const int64_t g0 = u * UNIT + (int64_t)tid * VEC;
                         if (g0 >= n) continue;
                         T xv[VEC], pv[VEC];
                         vld<T, VEC>(xi + g0, xv);
+                        if (pend || cf.f1 != T(0) || cf.fmode == 1) vld<T, VEC>(a.p + g0, pv);
+                        if (pend) {
+                            T wv[VEC];
+                            vld<T, VEC>(cf.prv[0] + g0, wv);
+#pragma unroll
+                            for (int v = 0; v < VEC; ++v) {
+                                xv[v] = fma(s.zxr[k6s], pv[v], xv[v]);
+                                pv[v] = fma(s.ppr[k6s], pv[v], wv[v]);
+                            }
+                        }
                         if (cf.fmode == 0) {
                             if (cf.f1 != T(0)) {
-                                vld<T, VEC>(a.p + g0, pv);
 #pragma unroll
                                 for (int v = 0; v < VEC; ++v) xv[v] = fma(cf.f1, pv[v], xv[v]);
                             }
@@ -1835,7 +1867,6 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
                             T vv[VEC];
                             vld<T, VEC>(cf.v0 + g0, vv);
                             if (cf.fmode == 1) {
-                                vld<T, VEC>(a.p + g0, pv);
 #pragma unroll
                                 for (int v = 0; v < VEC; ++v) {
                                     xv[v] = fma(cf.f1, pv[v], xv[v]);
@@ -1870,7 +1901,7 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
                 if (i + 1 >= L)
                     grp.template get_dots_warp<2 * L + 1>(a, s, (int)((i + 1 - L) % (L + 1)), s.raw2);
                 if ((tid & 31) == 0)
-                    scalar_step<T, L, kOolScalar, SC>(s, s.cfb[(i + 1) & 1], s.raw2, a, (int)(i + 1), rn, tau, budget,
+                    scalar_step<T, L, kOolScalar, SC, kPair>(s, s.cfb[(i + 1) & 1], s.raw2, a, (int)(i + 1), rn, tau, budget,
                                                   kc, kn);
                 __syncwarp();
             }
@@ -1887,7 +1918,9 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
             // the registers (and occupancy) a copy would take.
             using CoefRef = std::conditional_t<(RPT > 1), SweepCoef<T, L>, const Coef<T> &>;
             using StRef = std::conditional_t<(RPT > 1), StencilDesc, const StencilDesc &>;
+            using ZRef = std::conditional_t<(RPT > 1), T, const T &>;
             CoefRef C = cf;
+            const ZRef zx1 = s.zxr[k6s], pp1 = s.ppr[k6s];
             StRef st = a.st;
             const CsrDesc &csr = a.csr;
             T *const pvec = a.p;
@@ -1896,14 +1929,16 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
             const uint32_t usw = (uint32_t)(nsw * VEC * RPT);      // rows per sweep unit
             const uint32_t nunits_s = (tid < nsw) ? (nn + usw - 1) / usw : 0u;
             // Steady state -- every iteration of a segment after the first l + 1:
-            // the recurrences run, K6 updates p and x, z^(0)_{m-1} exists and the
-            // K5 operands follow a fixed pattern.  That case gets its own loop
-            // with those tests and the operand selection resolved at compile time.
-            const bool steady = C.mode == 1 && C.k6 == 2 && C.prev0 && !d2;
-            auto sweep = [&](auto steady_tag) {
+            // the recurrences run, z^(0)_{m-1} exists, K6 takes two steps of p and
+            // x (even m) or none (odd m), or one (kPair off), and the K5 operands follow a fixed
+            // pattern.  Those cases get their own loops with these tests and the
+            // operand selection resolved at compile time.
+            const bool steady = C.mode == 1 && C.k6 >= 2 && C.prev0 && !d2;
+            auto sweep = [&](auto steady_tag, auto k6_tag) {
                 constexpr bool S = decltype(steady_tag)::value;
+                constexpr int K6 = decltype(k6_tag)::value;   // 2, 3 or 4, 0: read from C
                 const bool rec = S || C.mode == 1;
-                const int k6 = S ? 2 : C.k6;
+                const int k6 = K6 ? K6 : C.k6;
                 const bool prev0 = S || C.prev0;
                 int since_flush = 0;
                 // 27-point tiles: the first unit's copies start here, each
@@ -1917,8 +1952,8 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
                     if (j == 0) return C.zl_prev;
                     if (j <= L) return C.cur[j - 1];
                     if (j <= 2 * L) return C.prv[j - 1 - L];
-                    if (j == 2 * L + 1) return pvec;
-                    if (j == 2 * L + 2) return static_cast<const T *>(xi);
+                    if (j == 2 * L + 1) return k6 != 3 ? pvec : nullptr;
+                    if (j == 2 * L + 2) return k6 != 3 ? static_cast<const T *>(xi) : nullptr;
                     return static_cast<const T *>(csr.dinv);
                 };
                 // stage unit uu (if it exists) in buffer bb
@@ -2008,8 +2043,10 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
                                     cur[r][k][0] = tile.vec(tb, 1 + k)[t];
                                     pk[r][k][0] = tile.vec(tb, 1 + L + k)[t];
                                 }
-                                pv[r][0] = tile.vec(tb, 2 * L + 1)[t];
-                                xv[r][0] = tile.vec(tb, 2 * L + 2)[t];
+                                if (k6 != 3) {
+                                    pv[r][0] = tile.vec(tb, 2 * L + 1)[t];
+                                    xv[r][0] = tile.vec(tb, 2 * L + 2)[t];
+                                }
                                 if constexpr (op_is_jacobi(OP)) {
                                     c[r][0] = tile.vec(tb, 2 * L + 3)[t];   // 1 / a_gg for now
                                     dg[r] = tile.diag(tb, t);                // a_gg: the diagonal slot
@@ -2044,7 +2081,7 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
                                 }
                             }
                         }
-                        if (k6 == 2) {
+                        if (k6 == 2 || k6 == 4) {
                             vld<T, VEC>(pvec + g0[r], pv[r]);
                             vld<T, VEC>(xi + g0[r], xv[r]);
                         }
@@ -2106,7 +2143,13 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
                         if (k6 == 1) {
 #pragma unroll
                             for (int v = 0; v < VEC; ++v) pv[r][v] = cur[r][0][v];
-                        } else if (k6 == 2) {
+                        } else if (k6 != 0 && k6 != 3) {
+                            if (kPair)
+#pragma unroll
+                                for (int v = 0; v < VEC; ++v) {
+                                    xv[r][v] = fma(zx1, pv[r][v], xv[r][v]);
+                                    pv[r][v] = fma(pp1, pv[r][v], pk[r][0][v]);
+                                }
 #pragma unroll
                             for (int v = 0; v < VEC; ++v) {
                                 xv[r][v] = fma(C.zx, pv[r][v], xv[r][v]);
@@ -2121,8 +2164,8 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
 #pragma unroll
                             for (int k = 0; k < L; ++k) vst<T, VEC>(C.nw[k] + g0[r], nw[k]);
                         }
-                        if (k6 >= 1) vst<T, VEC>(pvec + g0[r], pv[r]);
-                        if (k6 == 2) vst<T, VEC>(xi + g0[r], xv[r]);
+                        if (k6 != 0 && k6 != 3) vst<T, VEC>(pvec + g0[r], pv[r]);
+                        if (k6 == 2 || k6 == 4) vst<T, VEC>(xi + g0[r], xv[r]);
                         // -- K5: partial dot products with u_{i+1} = M z^(l)_{i+1}
                         // (M = I: z^(l)_{i+1} itself)
                         T uM[VEC];
@@ -2154,8 +2197,15 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
                     tb = (tb + 1) % Tile::NB;
                 }
             };
-            if (steady) sweep(std::true_type{});
-            else sweep(std::false_type{});
+            // (one loop for both where a sweep is short: its instructions are
+            // fetched anew in every launch, and a second loop's cost more than
+            // the test)
+            constexpr bool kSplit = std::is_same<Grp, BlockGroup<T>>::value || VEC > 1 || kTile;
+            if (!steady) sweep(std::false_type{}, std::integral_constant<int, 0>{});
+            else if constexpr (!kPair) sweep(std::true_type{}, std::integral_constant<int, 4>{});
+            else if constexpr (!kSplit) sweep(std::true_type{}, std::integral_constant<int, 0>{});
+            else if (C.k6 == 2) sweep(std::true_type{}, std::integral_constant<int, 2>{});
+            else sweep(std::true_type{}, std::integral_constant<int, 3>{});
             double acc[2 * L + 1];
 #pragma unroll
             for (int q = 0; q <= 2 * L; ++q) {
@@ -2182,7 +2232,7 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
                     if (i + 1 >= L)
                         grp.template get_dots_warp<2 * L + 1>(a, s, (int)((i + 1 - L) % (L + 1)), s.raw);
                     if (tid == 0)
-                        scalar_step<T, L, kOolScalar, SC>(s, s.cfb[(i + 1) & 1], s.raw, a, (int)(i + 1), rn, tau,
+                        scalar_step<T, L, kOolScalar, SC, kPair>(s, s.cfb[(i + 1) & 1], s.raw, a, (int)(i + 1), rn, tau,
                                                       budget, kc, kn);
                 }
                 __syncthreads();
