@@ -472,7 +472,8 @@ template <typename T>
 static plcg_status build_solve(const plcg_matrix *A, const double *b, double *x,
                                const plcg_params *prm, const double *sigma, int max_ctas,
                                char *base, SolveArgs<T> *args, const void **func_out,
-                               int64_t *P_out, int *per_sm_out, size_t *bytes, size_t *out_off)
+                               int64_t *P_out, int *per_sm_out, size_t *bytes, size_t *out_off,
+                               bool server = false)
 {
     const int64_t n = A->n;
     const int l = prm->l;
@@ -523,11 +524,34 @@ static plcg_status build_solve(const plcg_matrix *A, const double *b, double *x,
     if (prm->grid_ctas > 0) P = std::min<int64_t>(P, prm->grid_ctas);
     if (max_ctas > 0) P = std::min<int64_t>(P, max_ctas);
     P = std::max<int64_t>(1, std::min<int64_t>(P, nunits));
+    // small and mid-sized stencil systems, p(l)-CG with l <= 3: every row's
+    // state in registers (resident.cuh), 32 rows per CTA at least, up to 4 per
+    // thread; a cluster limit raised above its default asks for the cluster
+    // path instead, and a server keeps the smaller footprint of the others
+    const int64_t cluster_rows = cg || l >= 2 ? g_cluster_rows : g_cluster_rows / 2;
+    int res_nsw = 0;
+    if (op == kOpStencil && !cg && l <= 3 && !prm->dots_2l1 && prm->grid_ctas == 0 && max_ctas == 0 && !server &&
+        !(g_cluster_rows > kClusterRowsDefault && n <= cluster_rows)) {
+        const int64_t ctas = std::min(A->num_sms, 32 * kResChunks);
+        for (int rows : {1, 2, 4}) {
+            if (n > ctas * kResSweep * rows) continue;
+            // 64 CTAs while that leaves them at most 160 rows each (an exchange
+            // among fewer is shorter: 2D 100^2 p(1)-CG 3.51 us per iteration with
+            // 105, 3.35 with 63, 3.69 with 40), then 160 rows, then every SM
+            const int64_t all = (n + 32 * rows * ctas - 1) / (32 * rows * ctas), few = (n + 2047) / 2048;
+            res_nsw = (int)(32 * std::max(all, std::min<int64_t>(few, 5)));
+            func = f32 ? kptr_resident_f32(l, rows) : kptr_resident_f64(l, rows);
+            P = (n + (int64_t)rows * res_nsw - 1) / ((int64_t)rows * res_nsw);
+            per_sm = 1;
+            dsmem = 0;
+            break;
+        }
+    }
     // small systems: one thread-block cluster holds the whole solve (its
     // barrier and distributed shared memory replace the grid barrier and the
     // partials in global memory)
     int cluster = 0;
-    if (n <= (cg || l >= 2 ? g_cluster_rows : g_cluster_rows / 2) && !c32 &&
+    if (n <= cluster_rows && !res_nsw && !c32 &&
         (op == kOpStencil || op == kOpCsr) && (cg || l <= 4) && prm->grid_ctas == 0) {
         const void *cf = f32 ? kptr_cluster_f32(op, vec, cg ? 0 : l, cg) : kptr_cluster_f64(op, vec, cg ? 0 : l, cg);
         const int c = cf ? cluster_size_for(cf, (int)std::min<int64_t>(16, nunits)) : 0;
@@ -574,6 +598,8 @@ static plcg_status build_solve(const plcg_matrix *A, const double *b, double *x,
     const int slots = cg ? 2 : (l + 1);
     const size_t o_part = off; off += align_up((size_t)slots * P * kMaxDots * sizeof(double), 256);
     const size_t o_npart = off; off += align_up((size_t)P * kNormSlots * sizeof(double), 256);
+    // the packets, the barrier counter and the result record: zeroed by every launch
+    const size_t o_pkt = off; off += res_nsw ? align_up((size_t)kResSlots * P * res_dots(l) * 16, 256) : 0;
     const size_t o_bar = off; off += 256;
     const size_t o_out = off; off += align_up(sizeof(DevResult), 256);
     *bytes = off;
@@ -614,6 +640,8 @@ static plcg_status build_solve(const plcg_matrix *A, const double *b, double *x,
     a.npart = reinterpret_cast<double *>(base + o_npart);
     a.bar = reinterpret_cast<unsigned *>(base + o_bar);
     a.out = reinterpret_cast<DevResult *>(base + o_out);
+    a.pkt = reinterpret_cast<unsigned long long *>(base + o_pkt);
+    a.res_nsw = res_nsw;
     a.method = cg ? 1 : 0;
     a.l = l;
     for (int k = 0; k < l && k < kMaxL; ++k) a.sigma[k] = sigma[k];
@@ -652,8 +680,7 @@ static plcg_status launch_built(const SolveArgs<T> &a0, const void *func, int64_
                                 cudaStream_t stream)
 {
     SolveArgs<T> a = a0;
-    CUDA_TRY(cudaMemsetAsync(a.bar, 0, 256, stream));
-    CUDA_TRY(cudaMemsetAsync(a.out, 0, sizeof(DevResult), stream));
+    CUDA_TRY(cudaMemsetAsync(a.pkt, 0, reinterpret_cast<char *>(a.out + 1) - reinterpret_cast<char *>(a.pkt), stream));
     g_last_launch.kernel = (uint64_t)reinterpret_cast<uintptr_t>(func);
     g_last_launch.grid_ctas = (int)P;
     g_last_launch.dyn_smem = a.dsmem;
@@ -679,7 +706,7 @@ static plcg_status launch_built(const SolveArgs<T> &a0, const void *func, int64_
         cfg.numAttrs = 1;
         CUDA_TRY(cudaLaunchKernelExC(&cfg, func, args));
     } else {
-        CUDA_TRY(cudaLaunchCooperativeKernel(func, dim3((unsigned)P), dim3(kBlock), args, a.dsmem, stream));
+        CUDA_TRY(cudaLaunchCooperativeKernel(func, dim3((unsigned)P), dim3(a.res_nsw ? kResBlock : kBlock), args, a.dsmem, stream));
     }
     return PLCG_OK;
 }
@@ -1373,7 +1400,7 @@ static plcg_status server_launch(plcg_server *S, ServerReq &q)
     int per_sm = 0;
     size_t bytes = 0, o_out = 0;
     plcg_status s = build_solve<T>(q.A, q.b, q.x, &q.prm, q.sigma, (int)q.P, static_cast<char *>(ws),
-                                   &a, &func, &P, &per_sm, &bytes, &o_out);
+                                   &a, &func, &P, &per_sm, &bytes, &o_out, true);
     if (s == PLCG_OK) {
         CUDA_TRY(cudaEventRecord(S->ev0[q.slot], st));
         s = launch_built<T>(a, func, P, st);
@@ -1531,10 +1558,10 @@ extern "C" plcg_status plcg_submit(plcg_server *S, plcg_matrix *A, const double 
     size_t bytes = 0, o_out = 0;
     if (prm->prec != PLCG_FP32_FP64DOT) {
         SolveArgs<double> a;
-        st = build_solve<double>(A, b, x, &q->prm, q->sigma, 0, nullptr, &a, &func, &P, &per_sm, &bytes, &o_out);
+        st = build_solve<double>(A, b, x, &q->prm, q->sigma, 0, nullptr, &a, &func, &P, &per_sm, &bytes, &o_out, true);
     } else {
         SolveArgs<float> a;
-        st = build_solve<float>(A, b, x, &q->prm, q->sigma, 0, nullptr, &a, &func, &P, &per_sm, &bytes, &o_out);
+        st = build_solve<float>(A, b, x, &q->prm, q->sigma, 0, nullptr, &a, &func, &P, &per_sm, &bytes, &o_out, true);
     }
     if (st != PLCG_OK) return st;
     const int cap = std::max(1, (per_sm * S->num_sms) / 2);
@@ -1543,10 +1570,10 @@ extern "C" plcg_status plcg_submit(plcg_server *S, plcg_matrix *A, const double 
     // recompute the byte count for the capped grid (partials scale with P)
     if (prm->prec != PLCG_FP32_FP64DOT) {
         SolveArgs<double> a;
-        st = build_solve<double>(A, b, x, &q->prm, q->sigma, (int)q->P, nullptr, &a, &func, &P, &per_sm, &bytes, &o_out);
+        st = build_solve<double>(A, b, x, &q->prm, q->sigma, (int)q->P, nullptr, &a, &func, &P, &per_sm, &bytes, &o_out, true);
     } else {
         SolveArgs<float> a;
-        st = build_solve<float>(A, b, x, &q->prm, q->sigma, (int)q->P, nullptr, &a, &func, &P, &per_sm, &bytes, &o_out);
+        st = build_solve<float>(A, b, x, &q->prm, q->sigma, (int)q->P, nullptr, &a, &func, &P, &per_sm, &bytes, &o_out, true);
     }
     if (st != PLCG_OK) return st;
     q->bytes = bytes;

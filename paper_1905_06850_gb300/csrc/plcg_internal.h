@@ -122,6 +122,8 @@ struct SolveArgs {
                               // at least as many after every ring vector)
     int nring;                // ring vectors in zring
     int stage;                // CSR kernels: stage each unit's entries (rows long enough to pay)
+    unsigned long long *pkt;  // register-resident solver: the exchange packets (zeroed per launch)
+    int res_nsw;              // ... and its sweeping threads per CTA (0: not that solver)
     double *trace;            // CG: alpha_k, beta_k of the first segment (spectrum estimates), or null
     int trace_cap;            // pairs trace can hold
 };
@@ -197,6 +199,16 @@ constexpr unsigned csr_stage_bytes(unsigned value_bytes)
 {
     return 128u + 8u * (unsigned)kCsrStageWarpCap * (4u + value_bytes);
 }
+
+// The register-resident solver (resident.cuh): threads per CTA, of which the
+// first two warps do the exchanges and the scalars and up to kResSweep sweep;
+// its packets, [kResSlots exchanges][CTA][res_dots(l) doubles of 16 bytes];
+// and the chunks of 32 CTAs, one lane each, that an exchange covers.
+constexpr int kResBlock = 512;
+constexpr int kResSweep = kResBlock - 64;
+constexpr int kResSlots = 8;
+PLCG_HD constexpr int res_dots(int l) { return l == 1 ? 2 : 4; }
+constexpr int kResChunks = 5;
 
 // One system of a batched solve (stencil operators only).
 struct BatchSys {

@@ -45,6 +45,10 @@ const void *kptr_f32_v27j(int l, bool cg);
 // l = 1..4 or classic CG); nullptr when not instantiated.
 const void *kptr_cluster_f64(int op, int vec, int l, bool cg);
 const void *kptr_cluster_f32(int op, int vec, int l, bool cg);
+// The register-resident solver of small stencil systems (l = 1..3; 1, 2 or 4
+// rows per thread); nullptr when not instantiated.
+const void *kptr_resident_f64(int l, int rows);
+const void *kptr_resident_f32(int l, int rows);
 const void *kptr_m_csr(int l, bool cg, bool sc);
 const void *kptr_m_csrj(int l, bool cg, bool sc);
 const void *kptr_m_v27(int l, bool cg, bool sc);

@@ -135,7 +135,8 @@ CLUSTER_ROWS_DEFAULT = 12288
 def set_cluster_rows(max_rows: int = CLUSTER_ROWS_DEFAULT):
     """plcg_set_cluster_rows: small systems run on one thread-block cluster
     (p(l >= 2)-CG and CG up to max_rows rows, p(1)-CG up to half; 0: never;
-    no argument: the library's default)."""
+    no argument: the library's default, with which p(1..3)-CG on stencils
+    runs on the register-resident solver instead)."""
     _check(load().plcg_set_cluster_rows(int(max_rows)))
 
 
