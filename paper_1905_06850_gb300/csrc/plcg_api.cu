@@ -509,7 +509,8 @@ static plcg_status build_solve(const plcg_matrix *A, const double *b, double *x,
     unsigned dsmem = (op_is_csr(op) && (!cg || f32)) ? csr_stage_bytes(value_bytes)
                    : (op_is_var27(op) && f32 && !c32)
                        ? (cg ? v27_tile_bytes_cg((unsigned)sizeof(T))
-                             : v27_tile_bytes((unsigned)sizeof(T), l, op_is_jacobi(op))) : 0u;
+                             : v27_tile_bytes((unsigned)sizeof(T), l, op_is_jacobi(op)))
+                   : (!cg && pipe_used(op, vec, l)) ? 2u * pipe_stage_bytes(l) : 0u;
     if (dsmem) {
         CUDA_TRY(cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dsmem));
         CUDA_TRY(cudaFuncSetAttribute(func, cudaFuncAttributePreferredSharedMemoryCarveout,

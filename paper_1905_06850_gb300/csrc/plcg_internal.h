@@ -190,6 +190,16 @@ constexpr unsigned v27_tile_bytes_cg(unsigned value_bytes)
     return v27_tile_bytes_nv(value_bytes, 0, kV27StageBwdCg);
 }
 
+// Operands of a stencil sweep that are copied a unit ahead (StencilPipe):
+// stencils with 16 bytes of rows per thread, l <= 2 (two CTAs per SM hold
+// their two stages of 16-byte slots and, per warp, two edge slots).
+PLCG_HD constexpr bool pipe_used(int op, int vec, int l) { return op == kOpStencil && vec > 1 && l <= 2; }
+PLCG_HD constexpr int pipe_ops(int l) { return 8 + 2 * l; }
+PLCG_HD constexpr unsigned pipe_stage_bytes(int l)
+{
+    return (unsigned)pipe_ops(l) * (unsigned)kBlock * 16u + (unsigned)(kBlock / 32) * 16u;
+}
+
 // CSR entries (column index + value) each warp of a CSR kernel stages in
 // shared memory for its 32 rows of a sweep unit; warps whose rows have more
 // entries read them from global memory.  Layout of the dynamic shared

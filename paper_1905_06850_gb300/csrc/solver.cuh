@@ -766,6 +766,134 @@ struct Var27Tile {
     }
 };
 
+// ------------------------------------------------------------------------
+// Asynchronous copies of a stencil sweep's operands (cp.async): each thread
+// copies the 16 bytes of every operand of its rows -- the row group itself, its
+// y and z neighbours, and the streamed vectors -- into slots of its own, a unit
+// ahead of the one it computes, so that a sweep has two units of loads in
+// flight without the registers to hold them.  A neighbour outside the grid is
+// filled with zeros; the x neighbours come from the adjacent lanes, at a
+// warp's edges from two slots of its own.  Slots are private to a thread (no
+// barrier), and a slot is filled again only after its values were used.  The
+// sweep was bound by the latency of its loads (24 warps per SM, one unit each
+// in flight): 3D 256^3 FP32 p(1)-CG 107.5 -> 95.2 us per iteration with 16 warps
+// and two units, FP64 p(1) 263.6 -> 255.8 (bound by the FP64 units: 213), 128^3
+// FP32 p(2) 23.6 -> 18.8.  Three CTAs per SM with 80 registers and p and x
+// loaded directly spill: FP64 256^3 279.8.
+// ------------------------------------------------------------------------
+__device__ __forceinline__ void cp_async_ca16(uint32_t dst, const void *src, bool on)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(on ? 16 : 0) : "memory");
+}
+
+__device__ __forceinline__ void cp_async_cg16(uint32_t dst, const void *src, bool on)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(on ? 16 : 0) : "memory");
+}
+
+template <int N>
+__device__ __forceinline__ void cp_async_ca(uint32_t dst, const void *src, bool on)   // N = 4 or 8 bytes
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(dst), "l"(src), "n"(N), "r"(on ? N : 0)
+                 : "memory");
+}
+
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+template <typename T, int L, int VEC>
+struct StencilPipe {
+    static constexpr int kOps = pipe_ops(L);          // c, y-, y+, z-, z+, z_{i-1}, z^(k), previous z^(k), p, x
+    static constexpr uint32_t kStage = pipe_stage_bytes(L);
+    uint32_t base;                                    // this thread's slot of operand 0, stage 0
+    uint32_t edge;                                    // this warp's edge slots, stage 0
+    __device__ __forceinline__ explicit StencilPipe(unsigned char *dsm)
+        : base(smem_addr(dsm) + threadIdx.x * 16u),
+          edge(smem_addr(dsm) + (uint32_t)kOps * kBlock * 16u + (threadIdx.x >> 5) * 16u)
+    {
+    }
+    __device__ __forceinline__ uint32_t slot(int stage, int op) const
+    {
+        return base + (uint32_t)stage * kStage + (uint32_t)op * (kBlock * 16u);
+    }
+    template <class V>
+    __device__ __forceinline__ void get(int stage, int op, V (&o)[VEC]) const
+    {
+        if constexpr (sizeof(V) == 8) {
+            asm volatile("ld.shared.v2.f64 {%0, %1}, [%2];" : "=d"(o[0]), "=d"(o[1]) : "r"(slot(stage, op)) : "memory");
+        } else {
+            asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                         : "=f"(o[0]), "=f"(o[1]), "=f"(o[2]), "=f"(o[3]) : "r"(slot(stage, op)) : "memory");
+        }
+    }
+    __device__ __forceinline__ T get_edge(int stage, int side) const
+    {
+        T v;
+        const uint32_t a = edge + (uint32_t)stage * kStage + (uint32_t)side * 8u;
+        if constexpr (sizeof(T) == 8) asm volatile("ld.shared.f64 %0, [%1];" : "=d"(v) : "r"(a) : "memory");
+        else asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+        return v;
+    }
+    // Start the copies of z's part for the row group g0 (in: it exists);
+    // returns bits 0, 1: it has a left, a right neighbour.
+    __device__ __forceinline__ uint32_t issue_z(int stage, const StencilDesc &st, const T *z, uint32_t g0, bool in) const
+    {
+        const uint32_t nx = (uint32_t)st.nx, ny = (uint32_t)st.ny, nxy = nx * ny, lane = threadIdx.x & 31;
+        const uint32_t line = (__umulhi(g0, st.dnx.m) + g0) >> st.dnx.s;
+        const uint32_t x0 = g0 - line * nx;
+        const uint32_t zc = (__umulhi(line, st.dny.m) + line) >> st.dny.s;
+        const uint32_t y = line - zc * ny;
+        const bool l = in && x0 > 0, r = in && x0 + VEC < nx;
+        const bool ym = in && y > 0, yp = in && y + 1 < ny;
+        cp_async_ca16(slot(stage, 0), z + (in ? g0 : 0u), in);
+        cp_async_ca16(slot(stage, 1), z + (ym ? g0 - nx : 0u), ym);
+        cp_async_ca16(slot(stage, 2), z + (yp ? g0 + nx : 0u), yp);
+        if (st.dim == 3) {
+            const bool zm = in && zc > 0, zp = in && zc + 1 < (uint32_t)st.nz;
+            cp_async_ca16(slot(stage, 3), z + (zm ? g0 - nxy : 0u), zm);
+            cp_async_ca16(slot(stage, 4), z + (zp ? g0 + nxy : 0u), zp);
+        }
+        const uint32_t ea = edge + (uint32_t)stage * kStage;
+        if (lane == 0) cp_async_ca<(int)sizeof(T)>(ea, z + (l ? g0 - 1 : 0u), l);
+        if (lane == 31) cp_async_ca<(int)sizeof(T)>(ea + 8u, z + (r ? g0 + VEC : 0u), r);
+        return (l ? 1u : 0u) | (r ? 2u : 0u);
+    }
+    // Centre values and neighbour sums of the staged row group (whole warps).
+    __device__ __forceinline__ void parts(int stage, bool three, uint32_t lr, T (&c)[VEC], T (&nb)[VEC]) const
+    {
+        const uint32_t lane = threadIdx.x & 31;
+        get(stage, 0, c);
+        const T lf = __shfl_up_sync(0xffffffffu, c[VEC - 1], 1), rt = __shfl_down_sync(0xffffffffu, c[0], 1);
+        const T left = (lr & 1u) ? (lane == 0 ? get_edge(stage, 0) : lf) : T(0);
+        const T right = (lr & 2u) ? (lane == 31 ? get_edge(stage, 1) : rt) : T(0);
+        T ym[VEC], yp[VEC], zm[VEC], zp[VEC];
+        get(stage, 1, ym);
+        get(stage, 2, yp);
+        if (three) {
+            get(stage, 3, zm);
+            get(stage, 4, zp);
+        }
+#pragma unroll
+        for (int v = 0; v < VEC; ++v) {
+            const T a = (v > 0) ? c[v - 1] : left, b = (v < VEC - 1) ? c[v + 1] : right;
+            if constexpr (sizeof(T) == 8) {
+                if (three) {
+                    const double x[6] = {a, b, ym[v], yp[v], zm[v], zp[v]};
+                    nb[v] = fx_sum(x);
+                } else {
+                    const double x[4] = {a, b, ym[v], yp[v]};
+                    nb[v] = fx_sum(x);
+                }
+            } else {
+                nb[v] = ((a + b) + ym[v]) + yp[v];
+                if (three) nb[v] = (nb[v] + zm[v]) + zp[v];
+            }
+        }
+    }
+};
+
 // Per-warp staging of CSR entries in shared memory (dynamic shared memory,
 // layout in plcg_internal.h).  Every warp stages the entries of its own 32
 // rows of a sweep unit -- a contiguous range, since the rows are -- with one
@@ -1729,6 +1857,9 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
             }
         }
     }
+    // stencils with 16 bytes of rows per thread on the whole grid: the steady
+    // sweep's operands are copied a unit ahead (StencilPipe)
+    constexpr bool kPipe = pipe_used(OP, VEC, L) && std::is_same<Grp, GridGroup<T>>::value && RPT == 1;
     const int64_t n = a.n;
     const int64_t nunits = (n + UNIT - 1) / UNIT;
     const int tid = threadIdx.x;
@@ -1927,7 +2058,10 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
             DotAcc<T, VEC> dac[2 * L + 1];
             const uint32_t nn = (uint32_t)n;                      // n < 2^31
             const uint32_t usw = (uint32_t)(nsw * VEC * RPT);      // rows per sweep unit
-            const uint32_t nunits_s = (tid < nsw) ? (nn + usw - 1) / usw : 0u;
+            // the CTA's units: ucnt of them, udir apart
+            const uint32_t nunits_s = (nn + usw - 1) / usw, u0 = (uint32_t)grp.unit0(), us = (uint32_t)grp.ustep();
+            const uint32_t ucnt = (tid < nsw && u0 < nunits_s) ? (nunits_s - u0 + us - 1) / us : 0u;
+            const uint32_t ufirst = u0, udir = us;
             // Steady state -- every iteration of a segment after the first l + 1:
             // the recurrences run, z^(0)_{m-1} exists, K6 takes two steps of p and
             // x (even m) or none (odd m), or one (kPair off), and the K5 operands follow a fixed
@@ -1956,9 +2090,10 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
                     if (j == 2 * L + 2) return k6 != 3 ? static_cast<const T *>(xi) : nullptr;
                     return static_cast<const T *>(csr.dinv);
                 };
-                // stage unit uu (if it exists) in buffer bb
-                auto tile_issue = [&](int bb, uint32_t uu) {
-                    const bool more = uu < nunits_s;
+                // stage it in buffer bb
+                auto tile_issue = [&](int bb, uint32_t j) {   // the sweep's unit number j, if it exists
+                    const bool more = j < ucnt;
+                    const uint32_t uu = ufirst + j * udir;
                     const bool on = tile.issue(bb, more, more ? uu * usw : 0u, more ? min(uu * usw + usw, nn) : 0u,
                                                nsw);
                     stg_q = (stg_q & ~(1u << bb)) | ((on ? 1u : 0u) << bb);
@@ -1972,16 +2107,43 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
                     if (Tile::issues(nsw)) fence_proxy_async_all();
                     tile.prepare(SV, vsrc, st, static_cast<const T *>(csr.val), csr.stride, tclo, tchi, C.zl_cur,
                                  a.ws_lo, a.ws_hi, nsw);
-                    if ((uint32_t)grp.unit0() < nunits_s)
-                        for (int bb = 0; bb < Tile::NB - 1; ++bb)
-                            tile_issue(bb, (uint32_t)grp.unit0() + (uint32_t)bb * (uint32_t)grp.ustep());
+                    if (ucnt > 0)
+                        for (int bb = 0; bb < Tile::NB - 1; ++bb) tile_issue(bb, (uint32_t)bb);
                 }
+                constexpr bool kPiped = kPipe && S;
+                StencilPipe<T, kPipe ? L : 1, VEC> pipe(plcg_dsm);
+                uint32_t lr0 = 0, lr1 = 0;   // the staged units' x neighbours (this unit, the next)
+                auto pipe_issue = [&](int stage, uint32_t j) -> uint32_t {   // the sweep's unit number j
+                    uint32_t lr = 0;
+                    if constexpr (kPiped) {
+                        const uint32_t g = (ufirst + j * udir) * usw + (uint32_t)tid * VEC;
+                        const bool in = j < ucnt && g < nn;
+                        const uint32_t gs = in ? g : 0u;
+                        if (j < ucnt) {
+                            lr = pipe.issue_z(stage, st, C.zl_cur, gs, in);
+                            cp_async_cg16(pipe.slot(stage, 5), C.zl_prev + gs, in);
+#pragma unroll
+                            for (int k = 0; k < L; ++k) {
+                                cp_async_cg16(pipe.slot(stage, 6 + k), C.cur[k] + gs, in);
+                                cp_async_cg16(pipe.slot(stage, 6 + L + k), C.prv[k] + gs, in);
+                            }
+                            if (k6 != 3) {
+                                cp_async_cg16(pipe.slot(stage, 6 + 2 * L), pvec + gs, in);
+                                cp_async_cg16(pipe.slot(stage, 7 + 2 * L), static_cast<const T *>(xi) + gs, in);
+                            }
+                        }
+                        cp_async_commit();
+                    }
+                    return lr;
+                };
+                lr0 = pipe_issue(0, 0);
+                lr1 = pipe_issue(1, 1);
                 typename CsrStage<CT>::Rows rp_next{0, 0};   // the warp's next unit's row pointers
                 if constexpr (kStage) {
-                    const uint32_t w0 = (uint32_t)grp.unit0() * usw + (uint32_t)(tid & ~31);
-                    if (a.stage && w0 < nn) rp_next = CsrStage<CT>::rows_load(csr, w0, min(w0 + 32u, nn));
+                    const uint32_t w0 = ufirst * usw + (uint32_t)(tid & ~31);
+                    if (a.stage && ucnt > 0 && w0 < nn) rp_next = CsrStage<CT>::rows_load(csr, w0, min(w0 + 32u, nn));
                 }
-                for (uint32_t u = (uint32_t)grp.unit0(); u < nunits_s; u += (uint32_t)grp.ustep()) {
+                for (uint32_t j = 0, u = ufirst; j < ucnt; ++j, u += udir) {
                     uint32_t g0[RPT];
                     bool ok[RPT];
 #pragma unroll
@@ -1995,8 +2157,8 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
                         const uint32_t w0 = u * usw + (uint32_t)(tid & ~31);
                         if (a.stage && w0 < nn) {
                             const typename CsrStage<CT>::Rows rp = rp_next;
-                            const uint32_t wn = w0 + (uint32_t)grp.ustep() * usw;
-                            if (u + (uint32_t)grp.ustep() < nunits_s && wn < nn)
+                            const uint32_t wn = w0 + udir * usw;
+                            if (j + 1 < ucnt && wn < nn)
                                 rp_next = CsrStage<CT>::rows_load(csr, wn, min(wn + 32u, nn));
                             int64_t e0, e1;
                             CsrStage<CT>::rows_bounds(rp, &e0, &e1, &rs, &re);
@@ -2006,8 +2168,7 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
                     T bw[13];   // the tiled unit's backward coefficients (row g0[0])
                     if constexpr (kTile) {    // the copies NB - 1 units ahead; this unit's tile
                         stg = (stg_q >> tb) & 1u;
-                        tile_issue((tb + Tile::NB - 1) % Tile::NB,
-                                   u + (uint32_t)(Tile::NB - 1) * (uint32_t)grp.ustep());
+                        tile_issue((tb + Tile::NB - 1) % Tile::NB, j + (uint32_t)(Tile::NB - 1));
                         if (stg && ok[0]) tile.backward(g0[0], bw);
                         if (stg) tile.wait(tb, a.poll_limit, &a.out->abort);
                     }
@@ -2020,6 +2181,22 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
 #pragma unroll
                         for (int v = 0; v < VEC; ++v) zp[r][v] = T(0);
                         dg[r] = T(1);
+                        if constexpr (kPiped) {
+                            const int stage = (int)(j & 1u);
+                            cp_async_wait<1>();
+                            pipe.parts(stage, st.dim == 3, lr0, c[r], nb[r]);
+                            pipe.get(stage, 5, zp[r]);
+#pragma unroll
+                            for (int k = 0; k < L; ++k) {
+                                pipe.get(stage, 6 + k, cur[r][k]);
+                                pipe.get(stage, 6 + L + k, pk[r][k]);
+                            }
+                            if (k6 != 3) {
+                                pipe.get(stage, 6 + 2 * L, pv[r]);
+                                pipe.get(stage, 7 + 2 * L, xv[r]);
+                            }
+                            continue;
+                        }
                         if (!ok[r]) continue;
                         if constexpr (kStage) {   // K1 operands
                             if (stg) {
@@ -2194,8 +2371,13 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
                             if ((!D1 || q >= L) && (!S || steady_dot_src<L>(q) != 0)) dac[q].flush();   // dots in use
                         since_flush = 0;
                     }
+                    if constexpr (kPiped) {   // this unit's slots are free
+                        lr0 = lr1;
+                        lr1 = pipe_issue((int)(j & 1u), j + 2);
+                    }
                     tb = (tb + 1) % Tile::NB;
                 }
+                if constexpr (kPiped) cp_async_wait<0>();
             };
             // (one loop for both where a sweep is short: its instructions are
             // fetched anew in every launch, and a second loop's cost more than
@@ -2647,17 +2829,12 @@ finish:
 // Single-system kernels: the whole grid solves one system (cooperative
 // launch, so that every CTA is resident and the grid barrier can complete).
 // ------------------------------------------------------------------------
-// CTAs per SM the register budget is sized for: three for FP32 with l <= 2
-// and for the FP64 p(1)-CG stencil sweep with scaled bases and two rows per
-// thread (latency-bound once its neighbour sum runs on the integer units:
-// 3D 256^3 161.7 -> 138.5 ms at 85 registers with 72 bytes of spills,
-// against 128 registers at two CTAs per SM), two otherwise; the 27-point tiles' buffers (about 47 KB each) leave room
-// for one CTA per SM with four of them (two with two).
+// CTAs per SM the register budget is sized for: two for the sweeps whose
+// operands are copied ahead (their slots' shared memory), three for the other
+// FP32 sweeps with l <= 2, two otherwise; the 27-point tiles' buffers (about
+// 47 KB each) leave room for one CTA per SM with four of them (two with two).
 template <typename T, int L, int OP, bool SC = false, int VEC = 1>
-constexpr int kPlcgMinBlocks = (sizeof(T) == 4 && op_is_var27(OP)) ? 2
-                               : (sizeof(T) == 4 && L <= 2)       ? 3
-                               : (SC && L == 1 && OP == kOpStencil && VEC == 2) ? 3
-                                                                                : 2;
+constexpr int kPlcgMinBlocks = (sizeof(T) == 4 && L <= 2 && !op_is_var27(OP) && !pipe_used(OP, VEC, L)) ? 3 : 2;
 
 // CT: the stored type of the matrix values (T, or float under FP64 vectors:
 // the FP32-matrix path).
