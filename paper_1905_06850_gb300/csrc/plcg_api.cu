@@ -659,6 +659,14 @@ static plcg_status build_solve(const plcg_matrix *A, const double *b, double *x,
     a.lookahead = (!cg && l >= 2 && n < (int64_t(1) << 22)) ? 1 : 0;
     a.dsmem = dsmem;
     a.cluster = cluster;
+    // every other sweep backwards: the last part of one sweep is in L2 when the
+    // next starts there.  Measured with the vectors (and coefficients) an
+    // iteration touches at 50 .. 400 MB: 3D 128^3 FP32 p(3) 26.3 -> 22.9 us per
+    // iteration, FP64 p(1) 45.9 -> 44.5, 27-point 128^3 50.0 -> 49.2, 3D 256^3
+    // FP32 95.2 -> 93.4; at 805 MB (256^3 FP64 p(1)) 255.8 -> 259.5, and the
+    // staged CSR sweep loses at any size (107.0 -> 109.0)
+    const double touched = (double)n * (double)sizeof(T) * ((cg ? 4 : 2 * (l + 1) + 2) + (op_is_var27(op) ? 15 : 0));
+    a.snake = (!cg && touched <= 512e6) ? 1 : 0;
     // staging a warp's CSR entries pays when rows are long; short rows (the
     // diagonal toy has one entry) read them directly (measured)
     a.stage = (op_is_csr(op) && A->nnz >= 4 * n && !cluster) ? 1 : 0;

@@ -121,6 +121,7 @@ struct SolveArgs {
     int64_t halo;             // structured 27-point: zero elements before ring vector 0 (and
                               // at least as many after every ring vector)
     int nring;                // ring vectors in zring
+    int snake;                // every other sweep backwards
     int stage;                // CSR kernels: stage each unit's entries (rows long enough to pay)
     unsigned long long *pkt;  // register-resident solver: the exchange packets (zeroed per launch)
     int res_nsw;              // ... and its sweeping threads per CTA (0: not that solver)

@@ -1859,6 +1859,7 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
     }
     // stencils with 16 bytes of rows per thread on the whole grid: the steady
     // sweep's operands are copied a unit ahead (StencilPipe)
+    constexpr bool kSnake = std::is_same<Grp, GridGroup<T>>::value && !op_is_csr(OP) && !(SC && L == 1);
     constexpr bool kPipe = pipe_used(OP, VEC, L) && std::is_same<Grp, GridGroup<T>>::value && RPT == 1;
     const int64_t n = a.n;
     const int64_t nunits = (n + UNIT - 1) / UNIT;
@@ -2058,10 +2059,14 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
             DotAcc<T, VEC> dac[2 * L + 1];
             const uint32_t nn = (uint32_t)n;                      // n < 2^31
             const uint32_t usw = (uint32_t)(nsw * VEC * RPT);      // rows per sweep unit
-            // the CTA's units: ucnt of them, udir apart
+            // the CTA's units: ucnt of them, udir apart; every other sweep runs
+            // through them backwards where the solve's vectors are few times the
+            // L2's 126 MB (a.snake): what one sweep touched last the next one
+            // finds there
             const uint32_t nunits_s = (nn + usw - 1) / usw, u0 = (uint32_t)grp.unit0(), us = (uint32_t)grp.ustep();
             const uint32_t ucnt = (tid < nsw && u0 < nunits_s) ? (nunits_s - u0 + us - 1) / us : 0u;
-            const uint32_t ufirst = u0, udir = us;
+            const bool back = kSnake && a.snake && (i & 1) != 0;
+            const uint32_t ufirst = back ? u0 + (ucnt - 1) * us : u0, udir = back ? 0u - us : us;
             // Steady state -- every iteration of a segment after the first l + 1:
             // the recurrences run, z^(0)_{m-1} exists, K6 takes two steps of p and
             // x (even m) or none (odd m), or one (kPair off), and the K5 operands follow a fixed
