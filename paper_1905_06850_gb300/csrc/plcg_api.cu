@@ -66,6 +66,20 @@ extern "C" void plcg_debug_force_barrier_timeout(int on) { g_force_timeout = on 
 // and above ~2x10^4 rows the grid wins throughout.
 constexpr int64_t kClusterRowsDefault = 12288;
 constexpr int64_t kVec1Rows = 16384;
+// p(l)-CG with l <= 2 on stencils in 16-byte row groups: whether the sweep's
+// operands are copied a unit ahead (two CTAs per SM; the others have three, or
+// FP64 p(2) two).  us per iteration without and with: FP64 3D 128^3 p(1) 48.6
+// and 47.0, p(2) 57.8 and 56.9, 112^3 36.0 and 35.6, 41.7 and 41.8, but 96^3 p(2)
+// 27.0 and 29.2, 80^3 20.0 and 21.5, 20.3 and 22.3; FP32 p(2) 25.9 and 20.4 at
+// 128^3; FP32 p(1) 80^3 15.1 and 13.5, 112^3 17.8 and 17.6, 176^3 47.6 and 40.8,
+// but between (its vectors fit the L2, and the third CTA hides more of the
+// latency) 136 x 125 x 118 15.3 and 15.6, 128^3 20.0 and 20.4, 144^3 25.3 and 25.6.
+static bool copies_ahead(bool f32, int l, int64_t n)
+{
+    // (the 2 l + 1 dots' loop does not copy ahead)
+    if (!f32) return n >= (5 << 18);
+    return l != 1 || n < (7 << 18) || n >= (3 << 20);
+}
 static int64_t g_cluster_rows = kClusterRowsDefault;
 
 extern "C" plcg_status plcg_set_cluster_rows(int64_t max_rows)
@@ -467,13 +481,14 @@ static plcg_status ensure_ws(plcg_matrix *A, size_t bytes)
 
 // Layout of one solve's workspace and its kernel arguments.  With base ==
 // nullptr only the sizes are computed; *bytes is the workspace size and
-// *out_off the offset of the result record inside it.
+// *out_off the offset of the result record inside it.  pad_lines = false: no
+// padded lines (they take up to a fifth more workspace).
 template <typename T>
 static plcg_status build_solve(const plcg_matrix *A, const double *b, double *x,
                                const plcg_params *prm, const double *sigma, int max_ctas,
                                char *base, SolveArgs<T> *args, const void **func_out,
                                int64_t *P_out, int *per_sm_out, size_t *bytes, size_t *out_off,
-                               bool server = false)
+                               bool server = false, bool pad_lines = true)
 {
     const int64_t n = A->n;
     const int l = prm->l;
@@ -485,6 +500,14 @@ static plcg_status build_solve(const plcg_matrix *A, const double *b, double *x,
     const bool c32 = prm->prec == PLCG_FP32_MATRIX;
     if (c32 && f32) return fail(PLCG_ERR_INVALID, "internal: FP32 matrix path with FP32 vectors");
     const unsigned value_bytes = c32 ? 4u : (unsigned)sizeof(T);
+    // small and mid-sized stencil systems, p(l)-CG with l <= 3: every row's
+    // state in registers (resident.cuh), 32 rows per CTA at least, up to 4 per
+    // thread; a cluster limit raised above its default asks for the cluster
+    // path instead, and a server keeps the smaller footprint of the others
+    const int64_t cluster_rows = cg || l >= 2 ? g_cluster_rows : g_cluster_rows / 2;
+    const bool resident = op == kOpStencil && !cg && l <= 3 && !prm->dots_2l1 && prm->grid_ctas == 0 && max_ctas == 0 &&
+                          !server && !(g_cluster_rows > kClusterRowsDefault && n <= cluster_rows) &&
+                          n <= (int64_t)std::min(A->num_sms, 32 * kResChunks) * kResSweep * 4;
     // Stencil rows per thread: 16 bytes of a vector (rows in one x-line),
     // except FP64 systems of at most kVec1Rows rows, which take one row per
     // thread so that their FP64-bound sweep spreads over twice the SMs (or
@@ -492,16 +515,33 @@ static plcg_status build_solve(const plcg_matrix *A, const double *b, double *x,
     // p(1)-CG 7.11 -> 6.61 us per iteration, p(2) 6.54 -> 6.06, 2D 64^2 p(1)
     // 5.93 -> 5.16, 3D 20^3 p(1) 7.70 -> 6.78; from ~6*10^4 rows it costs
     // (3D 40^3 p(1) 8.9 -> 10.4 us), and the FP32 sweeps never gain
+    const int want = 16 / (int)sizeof(T);
     int vec = 1;
     if (op == kOpStencil) {
-        const int want = 16 / (int)sizeof(T);
         vec = (A->st.nx % want == 0 && !(sizeof(T) == 8 && n <= kVec1Rows)) ? want : 1;
     }
     // FP64 p(l)-CG on 2^19 rows or more: the scaled-basis kernel (one FP64
     // multiply per recurrence and row fewer; below that the longer scalar step
     // costs more) -- l <= 5 on the stencils, l = 1 on the stored operators
     const bool sc = !f32 && !cg && n >= (int64_t(1) << 19) && (l == 1 || (op == kOpStencil && l <= 5));
-    const void *func = kernel_ptr(f32, op, vec, cg ? 0 : l, cg, sc, c32);
+    // lines that are not whole vectors: the solver's vectors at a padded pitch,
+    // where the sweep is long (FP64: where the bases are scaled), instead of
+    // one row per thread.  3D 131^3 and 161^3, us per iteration, FP32 p(1)-CG
+    // 30 -> 22 and 59 -> 34, p(2) 34 -> 22 and 68 -> 38, p(3) 53 -> 29 and 95 ->
+    // 51; FP64 66 -> 51 and 113 -> 84, 75 -> 61 and 134 -> 104, 87 -> 74 and 155
+    // -> 126; 69^3 FP32 15.3 -> 13.4, 17.1 -> 13.8, 16.1 -> 16.2.
+    const int pitch = op == kOpStencil ? (int)align_up((size_t)A->st.nx, (size_t)want) : 0;
+    const bool pad = pad_lines && op == kOpStencil && vec == 1 && pitch != A->st.nx && A->st.nx >= 16 && !cg && l <= 3 &&
+                     !server && !resident && n > cluster_rows && (sc || (f32 && n >= (int64_t(1) << 18))) &&
+                     (int64_t)pitch * A->st.ny * A->st.nz < (int64_t(1) << 31);
+    const int64_t nv = pad ? (int64_t)pitch * A->st.ny * A->st.nz : n;   // rows of the solver's vectors
+    if (pad) vec = want;
+    // the sweep's operands copied a unit ahead
+    const bool ahead = op == kOpStencil && !cg && l <= 2 && vec > 1 &&
+                       (pad || (copies_ahead(f32, l, n) && !prm->dots_2l1));
+    const void *func = pad     ? kptr_st_pad(f32, l)
+                       : ahead ? kptr_st_ahead(f32, l)
+                               : kernel_ptr(f32, op, vec, cg ? 0 : l, cg, sc, c32);
     if (!func) return fail(PLCG_ERR_UNIMPL, "no kernel for prec=%d op=%d vec=%d l=%d", prm->prec, op, vec, l);
     // CSR kernels stage each unit's entries in dynamic shared memory (FP64
     // classic CG excepted, see cg_body); the FP32 27-point kernels stage
@@ -510,7 +550,7 @@ static plcg_status build_solve(const plcg_matrix *A, const double *b, double *x,
                    : (op_is_var27(op) && f32 && !c32)
                        ? (cg ? v27_tile_bytes_cg((unsigned)sizeof(T))
                              : v27_tile_bytes((unsigned)sizeof(T), l, op_is_jacobi(op)))
-                   : (!cg && pipe_used(op, vec, l)) ? 2u * pipe_stage_bytes(l) : 0u;
+                   : ahead ? 2u * pipe_stage_bytes(l) : 0u;
     if (dsmem) {
         CUDA_TRY(cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dsmem));
         CUDA_TRY(cudaFuncSetAttribute(func, cudaFuncAttributePreferredSharedMemoryCarveout,
@@ -520,19 +560,13 @@ static plcg_status build_solve(const plcg_matrix *A, const double *b, double *x,
     CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, func, kBlock, dsmem));
     if (per_sm < 1) return fail(PLCG_ERR_CUDA, "solver kernel cannot be resident");
     const int64_t unit = (int64_t)kBlock * vec;
-    const int64_t nunits = (n + unit - 1) / unit;
+    const int64_t nunits = (nv + unit - 1) / unit;
     int64_t P = (int64_t)per_sm * A->num_sms;
     if (prm->grid_ctas > 0) P = std::min<int64_t>(P, prm->grid_ctas);
     if (max_ctas > 0) P = std::min<int64_t>(P, max_ctas);
     P = std::max<int64_t>(1, std::min<int64_t>(P, nunits));
-    // small and mid-sized stencil systems, p(l)-CG with l <= 3: every row's
-    // state in registers (resident.cuh), 32 rows per CTA at least, up to 4 per
-    // thread; a cluster limit raised above its default asks for the cluster
-    // path instead, and a server keeps the smaller footprint of the others
-    const int64_t cluster_rows = cg || l >= 2 ? g_cluster_rows : g_cluster_rows / 2;
     int res_nsw = 0;
-    if (op == kOpStencil && !cg && l <= 3 && !prm->dots_2l1 && prm->grid_ctas == 0 && max_ctas == 0 && !server &&
-        !(g_cluster_rows > kClusterRowsDefault && n <= cluster_rows)) {
+    if (resident) {
         const int64_t ctas = std::min(A->num_sms, 32 * kResChunks);
         for (int rows : {1, 2, 4}) {
             if (n > ctas * kResSweep * rows) continue;
@@ -583,14 +617,14 @@ static plcg_status build_solve(const plcg_matrix *A, const double *b, double *x,
     }
     // ring vectors are packed with stride n (ring() indexes whole vectors);
     // 128-bit access needs n * sizeof(T) to be a multiple of 16
-    if (((size_t)n * sizeof(T)) % 16 != 0 && vec > 1)
+    if (((size_t)nv * sizeof(T)) % 16 != 0 && vec > 1)
         return fail(PLCG_ERR_INVALID, "internal: vector length not 16-byte aligned");
     // structured 27-point operators: a zero halo before the first ring vector
     // and at least one after every vector (the stride includes it), zeroed by
     // the kernel at the start of each solve, so that the tiles' z-line copies
     // stay inside the vector and zeros
     const int64_t halo = op_is_var27(op) ? v27_halo(A->st.nx, A->st.ny) : 0;
-    const size_t vbytes = align_up((size_t)(n + halo) * sizeof(T), 256);
+    const size_t vbytes = align_up((size_t)(nv + halo) * sizeof(T), 256);
     size_t off = 0;
     const size_t o_ring = off; off += (size_t)halo * sizeof(T) + vbytes * nvec;
     const size_t o_p = off; off += vbytes;
@@ -611,6 +645,12 @@ static plcg_status build_solve(const plcg_matrix *A, const double *b, double *x,
     if (!base) return PLCG_OK;
     a.n = n;
     a.st = A->st;
+    if (pad) {
+        a.st0 = A->st;
+        a.nxr = A->st.nx;
+        a.st.nx = pitch;
+        a.st.dnx = make_fastdiv((uint32_t)pitch);
+    }
     a.csr.rowptr = A->rowptr;
     a.csr.col = A->col;
     a.csr.val = A->val;
@@ -747,9 +787,14 @@ static plcg_status run_solve(plcg_matrix *A, const double *b, double *x, const p
     plcg_status st = build_solve<T>(A, b, x, prm, sigma, 0, nullptr, &a, &func, &P, &per_sm, &bytes, &o_out);
     if (st != PLCG_OK) return st;
     st = ensure_ws(A, bytes);
+    const bool pad_lines = st != PLCG_ERR_NOMEM;
+    if (!pad_lines) {   // without padded lines, if that needs less
+        st = build_solve<T>(A, b, x, prm, sigma, 0, nullptr, &a, &func, &P, &per_sm, &bytes, &o_out, false, false);
+        if (st == PLCG_OK) st = ensure_ws(A, bytes);
+    }
     if (st != PLCG_OK) return st;
     st = build_solve<T>(A, b, x, prm, sigma, 0, static_cast<char *>(A->ws.mem), &a, &func, &P,
-                        &per_sm, &bytes, &o_out);
+                        &per_sm, &bytes, &o_out, false, pad_lines);
     if (st != PLCG_OK) return st;
     a.trace = trace;
     a.trace_cap = trace_cap;
@@ -850,12 +895,15 @@ static plcg_status run_solve_fixed(const plcg_matrix *A, const double *b, double
     int per_sm = 0;
     size_t bytes = 0, o_out = 0;
     plcg_status st = build_solve<T>(A, b, x, prm, sigma, 0, nullptr, &a, &func, &P, &per_sm, &bytes, &o_out);
+    const bool pad_lines = st != PLCG_OK || bytes <= cap;
+    if (!pad_lines)
+        st = build_solve<T>(A, b, x, prm, sigma, 0, nullptr, &a, &func, &P, &per_sm, &bytes, &o_out, false, false);
     if (st != PLCG_OK) return st;
     if (bytes > cap)
         return fail(PLCG_ERR_INVALID,
                     "%s: this solve needs %zu bytes of scratch; the fixed no-allocation scratch holds %zu bytes "
                     "(use plcg_solve)", who, bytes, cap);
-    st = build_solve<T>(A, b, x, prm, sigma, 0, base, &a, &func, &P, &per_sm, &bytes, &o_out);
+    st = build_solve<T>(A, b, x, prm, sigma, 0, base, &a, &func, &P, &per_sm, &bytes, &o_out, false, pad_lines);
     if (st != PLCG_OK) return st;
     st = launch_built<T>(a, func, P, A->stream);
     if (st != PLCG_OK) return st;

@@ -122,6 +122,8 @@ struct SolveArgs {
                               // at least as many after every ring vector)
     int nring;                // ring vectors in zring
     int snake;                // every other sweep backwards
+    StencilDesc st0;          // padded lines: the caller's grid (st being the padded one)
+    int nxr;                  // ... and its line length
     int stage;                // CSR kernels: stage each unit's entries (rows long enough to pay)
     unsigned long long *pkt;  // register-resident solver: the exchange packets (zeroed per launch)
     int res_nsw;              // ... and its sweeping threads per CTA (0: not that solver)
@@ -194,7 +196,6 @@ constexpr unsigned v27_tile_bytes_cg(unsigned value_bytes)
 // Operands of a stencil sweep that are copied a unit ahead (StencilPipe):
 // stencils with 16 bytes of rows per thread, l <= 2 (two CTAs per SM hold
 // their two stages of 16-byte slots and, per warp, two edge slots).
-PLCG_HD constexpr bool pipe_used(int op, int vec, int l) { return op == kOpStencil && vec > 1 && l <= 2; }
 PLCG_HD constexpr int pipe_ops(int l) { return 8 + 2 * l; }
 PLCG_HD constexpr unsigned pipe_stage_bytes(int l)
 {

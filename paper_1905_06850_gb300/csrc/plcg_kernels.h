@@ -31,6 +31,8 @@ const void *batched_kernel_ptr_f64(int l, bool cg);
 const void *kptr_f64_st2(int l, bool cg, bool sc);
 const void *kptr_f64_st1(int l, bool cg, bool sc);
 const void *kptr_f64_stsc(int vec, int l);
+const void *kptr_st_ahead(bool f32, int l);
+const void *kptr_st_pad(bool f32, int l);
 const void *kptr_f64_csr(int l, bool cg, bool sc);
 const void *kptr_f32_st4(int l, bool cg);
 const void *kptr_f32_st1(int l, bool cg);

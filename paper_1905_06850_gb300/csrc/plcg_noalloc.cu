@@ -7,7 +7,7 @@
 // allocator.  This entry point runs the solve exactly as plcg_solve would
 // (the same argument checks, shifts, kernel, launch shape and kernel
 // arguments: solve_stencil_fixed in plcg_api.cu builds them with the code
-// plcg_solve uses), but the solver's scratch (basis rings, search direction,
+// plcg_solve uses, without padded lines where only they would not fit), but the solver's scratch (basis rings, search direction,
 // residual, reduction partials, barrier counter, result record) lives in one
 // file-scope __device__ array of kScratchBytes.  Every GPU that loads the
 // library holds that array until the process exits.

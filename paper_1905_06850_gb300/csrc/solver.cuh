@@ -837,8 +837,10 @@ struct StencilPipe {
         return v;
     }
     // Start the copies of z's part for the row group g0 (in: it exists);
-    // returns bits 0, 1: it has a left, a right neighbour.
-    __device__ __forceinline__ uint32_t issue_z(int stage, const StencilDesc &st, const T *z, uint32_t g0, bool in) const
+    // returns bits 0, 1: it has a left, a right neighbour, and (nxr rows per
+    // line, see PAD) the number of its rows in the line in the bits above.
+    __device__ __forceinline__ uint32_t issue_z(int stage, const StencilDesc &st, const T *z, uint32_t g0, bool in,
+                                                int nxr) const
     {
         const uint32_t nx = (uint32_t)st.nx, ny = (uint32_t)st.ny, nxy = nx * ny, lane = threadIdx.x & 31;
         const uint32_t line = (__umulhi(g0, st.dnx.m) + g0) >> st.dnx.s;
@@ -858,7 +860,7 @@ struct StencilPipe {
         const uint32_t ea = edge + (uint32_t)stage * kStage;
         if (lane == 0) cp_async_ca<(int)sizeof(T)>(ea, z + (l ? g0 - 1 : 0u), l);
         if (lane == 31) cp_async_ca<(int)sizeof(T)>(ea + 8u, z + (r ? g0 + VEC : 0u), r);
-        return (l ? 1u : 0u) | (r ? 2u : 0u);
+        return (l ? 1u : 0u) | (r ? 2u : 0u) | (uint32_t)max(0, min(VEC, nxr - (int)x0)) << 2;
     }
     // Centre values and neighbour sums of the staged row group (whole warps).
     __device__ __forceinline__ void parts(int stage, bool three, uint32_t lr, T (&c)[VEC], T (&nb)[VEC]) const
@@ -1436,10 +1438,19 @@ constexpr bool kScaledBases = (sizeof(T) == 8 && L <= 5);
 // instead of 3 l + 7 vector passes, the same operations on every row (3D 256^3
 // FP32 p(1)-CG 59.5 -> 55.1 ms, the batch of 4096 2D systems 51.2 -> 47.5 ms,
 // same bits).  Not where vector traffic is not the bound: the FP64 p(1)-CG
-// sweep with scaled bases (FP64 units; 122.7 -> 123.8 ms in pairs) and CSR
-// (matrix traffic; short solves lose by the longer loop).
-template <typename T, int L, int OP, bool SC>
-constexpr bool kPairK6 = !op_is_csr(OP) && !(SC && L == 1 && sizeof(T) == 8);
+// sweep (FP64 units; 3D 256^3 122.7 -> 123.8 ms in pairs, 80^3 19.8 -> 20.2 us
+// per iteration) and CSR
+// (matrix traffic; short solves lose by the longer loop), 27-point operators
+// (128^3 p(1)-CG 49.7 -> 49.5 us per iteration, 31 x 29 x 36 8.7 -> 8.85), one row per thread on
+// the grid (3D 131^3 FP32 p(1)-CG 29.6 -> 30.4 us per iteration: registers), nor
+// in one cluster or FP64 batches (521 systems of 38 .. 203, p(3)-CG 21.6 -> 21.9
+// ms: their vectors sit in L2).
+template <typename T, class Grp>
+constexpr bool kPairIn = std::is_same<Grp, GridGroup<T>>::value ||
+                         (sizeof(T) == 4 && !std::is_same<Grp, ClusterGroup<T>>::value);
+template <typename T, int L, int VEC, int OP, class Grp>
+constexpr bool kPairK6 = kPairIn<T, Grp> && OP == kOpStencil && !(L == 1 && sizeof(T) == 8) &&
+                         (VEC > 1 || !std::is_same<Grp, GridGroup<T>>::value);
 
 template <typename T, int L, bool SC, bool PAIR>
 __device__ __forceinline__ void scalar_step_body(Smem<T> &s, Coef<T> &cf, const double *raw,
@@ -1737,7 +1748,7 @@ struct DotAcc {
 // "Residual norm in p(l)-CG").  Units of kBlock * V64 rows.
 // ------------------------------------------------------------------------
 template <typename T, int VEC, int OP, class Grp, typename C = T>
-__device__ void residual_sweep(const SolveArgs<T> &a, Smem<T> &s, const Grp &grp)
+__device__ void residual_sweep(const SolveArgs<T> &a, const StencilDesc &st, Smem<T> &s, const Grp &grp)
 {
     constexpr int V64 = (VEC >= 2) ? 2 : 1;
     constexpr int UNIT = kBlock * V64;
@@ -1751,10 +1762,10 @@ __device__ void residual_sweep(const SolveArgs<T> &a, Smem<T> &s, const Grp &grp
         if (g0 >= (uint32_t)n) continue;
         double c[V64], w[V64], bv[V64];
         if constexpr (OP == kOpStencil) {
-            stencil_apply<double, V64>(a.st, cC, cO, ld, g0, c, w);
+            stencil_apply<double, V64>(st, cC, cO, ld, g0, c, w);
         } else if constexpr (op_is_var27(OP)) {
             c[0] = a.x[g0];
-            w[0] = var27_row<double, C>(a.st, static_cast<const C *>(a.csr.val), a.csr.stride, ld, g0);
+            w[0] = var27_row<double, C>(st, static_cast<const C *>(a.csr.val), a.csr.stride, ld, g0);
         } else {
             c[0] = a.x[g0];
             w[0] = csr_row<double, C>(a.csr, ld, g0);
@@ -1805,23 +1816,48 @@ __device__ __forceinline__ constexpr int steady_dot_src(int q)
     return q < L ? 0 : q == L ? 3 : q == 2 * L ? 2 : q == 2 * L - 1 ? 4 : q == 2 * L - 2 ? 5 : 1;
 }
 
+// Padded lines: how many rows of the vector group g0 are rows of the system,
+// and the first one's place in the caller's layout.
+struct PadRows {
+    int cnt;
+    uint32_t user;
+};
+
+template <bool PAD, int VEC, typename T>
+__device__ __forceinline__ PadRows pad_rows(const SolveArgs<T> &a, uint32_t g0)
+{
+    if constexpr (!PAD) return {VEC, g0};
+    const uint32_t line = (__umulhi(g0, a.st.dnx.m) + g0) >> a.st.dnx.s;
+    const int x0 = (int)(g0 - line * (uint32_t)a.st.nx);
+    return {max(0, min(VEC, a.nxr - x0)), line * (uint32_t)a.nxr + (uint32_t)x0};
+}
+
 // ------------------------------------------------------------------------
 // p(l)-CG: a whole solve on one group (grid or CTA).
 // ------------------------------------------------------------------------
 // D1: the l + 1 dots of Sec. 2.2 only (the 2l + 1 option compiled out: the
 // sweep then carries no accumulators for positions 0 .. l-1).
+// PIPE: the steady sweep's operands are copied a unit ahead (StencilPipe).
+// PAD (stencils on the whole grid): the solver's own vectors hold every grid
+// line at a pitch of whole VEC-row vectors (a.st.nx; the line's a.nxr rows,
+// then zeros), so that any line length takes vector loads; b, x and the
+// residual keep the caller's layout (a.st0, a.n rows), and the iterate is a
+// segment's correction in a.rc, as in FP32, in FP64 too.  Zeros stay zeros: the
+// sweep forms z^(l)'s new value with the padding masked, and every other
+// vector's padding from zeros.
 template <typename T, int L, int VEC, int OP, class Grp, int RPT = 1, bool SC = false, typename CT = T,
-          bool D1 = false>
+          bool D1 = false, bool PIPE = false, bool PAD = false>
 __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
 {
     const bool d2 = !D1 && a.dots_2l1;   // the 2l + 1 dots
     constexpr int UNIT = kBlock * VEC;
     constexpr bool kF32 = (sizeof(T) == 4);
-    constexpr bool kOolScalar = kF32 && std::is_same<Grp, GridGroup<T>>::value;
+    constexpr bool kGrid = std::is_same<Grp, GridGroup<T>>::value;
+    constexpr bool kOolScalar = kF32 && kGrid;
     // FP64 p(1)-CG keeps its bases scaled (see scalar_step_body): two FP64
     // multiplies per row fewer in the FP64-bound sweep
     constexpr bool kScaled = SC && kScaledBases<T, L>;
-    constexpr bool kPair = kPairK6<T, L, OP, SC>;
+    constexpr bool kPair = kPairK6<T, L, VEC, OP, Grp>;
     // CSR on the whole grid: each sweep unit's entries are bulk-copied into
     // shared memory (one contiguous range per unit) before its rows are read
     constexpr bool kStage = op_is_csr(OP) && std::is_same<Grp, GridGroup<T>>::value && RPT == 1;
@@ -1857,19 +1893,24 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
             }
         }
     }
-    // stencils with 16 bytes of rows per thread on the whole grid: the steady
-    // sweep's operands are copied a unit ahead (StencilPipe)
-    constexpr bool kSnake = std::is_same<Grp, GridGroup<T>>::value && !op_is_csr(OP) && !(SC && L == 1);
-    constexpr bool kPipe = pipe_used(OP, VEC, L) && std::is_same<Grp, GridGroup<T>>::value && RPT == 1;
-    const int64_t n = a.n;
+    // (the FP32 stencil sweeps at three CTAs per SM have no registers for it, nor
+    // have l > 4 and the FP64 27-point sweep; the FP64 p(1)-CG sweep gains nothing)
+    constexpr bool kSnake = kGrid && !(L == 1 && !kF32) &&
+                            (op_is_var27(OP) ? kF32 && L <= 2
+                                             : OP == kOpStencil && (PIPE || (!kF32 && VEC > 1 && L <= 4) || L == 3 || L == 4));
+    constexpr bool kPipe = PIPE;
+    static_assert(!PIPE || (OP == kOpStencil && VEC > 1 && kGrid && RPT == 1), "copies ahead: 16-byte rows");
+    static_assert(!PAD || (OP == kOpStencil && VEC > 1 && kGrid), "padded lines: stencils on the whole grid");
+    constexpr bool kCorr = kF32 || PAD;   // the iterate is a segment's correction of x
+    const int64_t n = PAD ? (int64_t)a.st.nx * a.st.ny * a.st.nz : a.n;   // rows of the solver's vectors
     const int64_t nunits = (n + UNIT - 1) / UNIT;
     const int tid = threadIdx.x;
     const T cC = (T)a.st.center, cO = (T)a.st.off;
     // (A z)_g = kc * c + kn * nb (see op_parts)
     const T kc = (OP == kOpStencil) ? cC : T(0), kn = (OP == kOpStencil) ? cO : T(1);
-    // xi: the iterate K6 updates (FP64 path: x itself; FP32 path: the inner
-    // correction d of the refinement step)
-    T *xi = kF32 ? a.rc : reinterpret_cast<T *>(a.x);
+    // xi: the iterate K6 updates (FP64 path: x itself; FP32 path and padded
+    // lines: the inner correction d of the refinement step)
+    T *xi = kCorr ? a.rc : reinterpret_cast<T *>(a.x);
 
     long long iters = 0, spmvs = 0, restarts = 0, refinements = 0, segments = 0;
     int last_end = kSegConverged;
@@ -1886,7 +1927,8 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
 
     for (;;) {
         // ---- true residual r = b - A x and its norm (Algorithm 1 initialization / the final check)
-        residual_sweep<T, VEC, OP, Grp, CT>(a, s, grp);
+        if constexpr (PAD) residual_sweep<T, 1, OP, Grp, CT>(a, a.st0, s, grp);
+        else residual_sweep<T, VEC, OP, Grp, CT>(a, a.st, s, grp);
         grp.put_norms(a, s);
         spmvs++;
         PLCG_SYNC();
@@ -1896,9 +1938,9 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
         last_rn = rn;
         if (normb == 0.0) {
             // b = 0: x = 0 is the solution
-            for (int64_t u = grp.unit0(); u * kBlock < n; u += grp.ustep()) {
+            for (int64_t u = grp.unit0(); u * kBlock < a.n; u += grp.ustep()) {
                 const int64_t g = u * kBlock + tid;
-                if (g < n) a.x[g] = 0.0;
+                if (g < a.n) a.x[g] = 0.0;
             }
             status = kStOk;
             break;
@@ -1928,16 +1970,19 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
                 const int64_t g0 = u * UNIT + (int64_t)tid * VEC;
                 if (g0 >= n) continue;
                 T z[VEC];
+                const PadRows pr = pad_rows<PAD, VEC>(a, (uint32_t)g0);
 #pragma unroll
                 for (int v = 0; v < VEC; ++v) {
-                    if constexpr (op_is_jacobi(OP))
+                    if constexpr (PAD)
+                        z[v] = v < pr.cnt ? (T)(a.r[pr.user + v] * inv) : T(0);
+                    else if constexpr (op_is_jacobi(OP))
                         z[v] = (T)(a.r[g0 + v] * __ldg(a.dinv64 + g0 + v) * inv);
                     else
                         z[v] = (T)(a.r[g0 + v] * inv);
                 }
 #pragma unroll
                 for (int k = 0; k <= L; ++k) vst<T, VEC>(ring(a, k, 0) + g0, z);
-                if constexpr (kF32) {
+                if constexpr (kCorr) {
                     T zero[VEC];
 #pragma unroll
                     for (int v = 0; v < VEC; ++v) zero[v] = T(0);
@@ -1964,6 +2009,12 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
         // l iterations later) with the local work, on one GPU.
         const bool la = (L >= 2) && a.lookahead;
         const int nsw = la ? kBlock - 32 : kBlock;   // threads that sweep
+        uint32_t ulast = 0;   // the CTA's last unit of a sweep, where sweeps run backwards
+        if constexpr (kSnake) {
+            const uint32_t rows = (uint32_t)(nsw * VEC * RPT), units = ((uint32_t)n + rows - 1) / rows;
+            const uint32_t u0 = (uint32_t)grp.unit0(), us = (uint32_t)grp.ustep();
+            ulast = u0 < units ? u0 + (units - 1 - u0) / us * us : u0;
+        }
         if (tid == 0) scalar_step<T, L, kOolScalar, SC, kPair>(s, s.cfb[0], s.raw, a, 0, rn, tau, budget, kc, kn);
         __syncthreads();
         for (long long i = 0;; ++i) {
@@ -1973,8 +2024,9 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
             if (cf.end >= 0) {
                 // ---- final vector update of the segment (a segment that ends on
                 // a non-finite scalar takes the outstanding step alone)
-                const bool pend = kPair && i >= L + 2 && ((i - L) & 1) == 0;   // step m - 1 is outstanding
-                if (cf.end != kSegNonfinite || (!kF32 && pend)) {
+                bool pend = false;
+                if constexpr (kPair) pend = i >= L + 2 && ((i - L) & 1) == 0;   // step m - 1 is outstanding
+                if (cf.end != kSegNonfinite || (!kF32 && (pend || PAD))) {
                     for (int64_t u = grp.unit0(); u < nunits; u += grp.ustep()) {
                         const int64_t g0 = u * UNIT + (int64_t)tid * VEC;
                         if (g0 >= n) continue;
@@ -2010,7 +2062,12 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
                                 for (int v = 0; v < VEC; ++v) xv[v] = fma(cf.f2, cf.pv * vv[v], xv[v]);
                             }
                         }
-                        if constexpr (kF32) {
+                        if constexpr (PAD) {
+                            const PadRows pr = pad_rows<PAD, VEC>(a, (uint32_t)g0);
+#pragma unroll
+                            for (int v = 0; v < VEC; ++v)
+                                if (v < pr.cnt) a.x[pr.user + v] += (double)xv[v];
+                        } else if constexpr (kF32) {
 #pragma unroll
                             for (int v = 0; v < VEC; ++v) a.x[g0 + v] += (double)xv[v];
                         } else {
@@ -2059,14 +2116,23 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
             DotAcc<T, VEC> dac[2 * L + 1];
             const uint32_t nn = (uint32_t)n;                      // n < 2^31
             const uint32_t usw = (uint32_t)(nsw * VEC * RPT);      // rows per sweep unit
-            // the CTA's units: ucnt of them, udir apart; every other sweep runs
-            // through them backwards where the solve's vectors are few times the
-            // L2's 126 MB (a.snake): what one sweep touched last the next one
-            // finds there
-            const uint32_t nunits_s = (nn + usw - 1) / usw, u0 = (uint32_t)grp.unit0(), us = (uint32_t)grp.ustep();
-            const uint32_t ucnt = (tid < nsw && u0 < nunits_s) ? (nunits_s - u0 + us - 1) / us : 0u;
+            // the CTA's units are udir apart, up to the first that is not below
+            // nunits_s (the one before number unit0() < ustep() wraps around);
+            // every other sweep runs through them backwards where the solve's
+            // vectors are few times the L2's 126 MB (a.snake): what one sweep
+            // touched last the next one finds there
+            const uint32_t nunits_s = (tid < nsw) ? (nn + usw - 1) / usw : 0u;
             const bool back = kSnake && a.snake && (i & 1) != 0;
-            const uint32_t ufirst = back ? u0 + (ucnt - 1) * us : u0, udir = back ? 0u - us : us;
+            // (computed where they are used: a register each would spill the
+            // kernels at their register limit)
+            auto ufirst = [&]() -> uint32_t {
+                if constexpr (kSnake) return back ? ulast : (uint32_t)grp.unit0();
+                else return (uint32_t)grp.unit0();
+            };
+            auto udir = [&]() -> uint32_t {
+                if constexpr (kSnake) return back ? 0u - (uint32_t)grp.ustep() : (uint32_t)grp.ustep();
+                else return (uint32_t)grp.ustep();
+            };
             // Steady state -- every iteration of a segment after the first l + 1:
             // the recurrences run, z^(0)_{m-1} exists, K6 takes two steps of p and
             // x (even m) or none (odd m), or one (kPair off), and the K5 operands follow a fixed
@@ -2095,10 +2161,9 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
                     if (j == 2 * L + 2) return k6 != 3 ? static_cast<const T *>(xi) : nullptr;
                     return static_cast<const T *>(csr.dinv);
                 };
-                // stage it in buffer bb
-                auto tile_issue = [&](int bb, uint32_t j) {   // the sweep's unit number j, if it exists
-                    const bool more = j < ucnt;
-                    const uint32_t uu = ufirst + j * udir;
+                // stage unit uu (if it exists) in buffer bb
+                auto tile_issue = [&](int bb, uint32_t uu) {
+                    const bool more = uu < nunits_s;
                     const bool on = tile.issue(bb, more, more ? uu * usw : 0u, more ? min(uu * usw + usw, nn) : 0u,
                                                nsw);
                     stg_q = (stg_q & ~(1u << bb)) | ((on ? 1u : 0u) << bb);
@@ -2112,20 +2177,20 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
                     if (Tile::issues(nsw)) fence_proxy_async_all();
                     tile.prepare(SV, vsrc, st, static_cast<const T *>(csr.val), csr.stride, tclo, tchi, C.zl_cur,
                                  a.ws_lo, a.ws_hi, nsw);
-                    if (ucnt > 0)
-                        for (int bb = 0; bb < Tile::NB - 1; ++bb) tile_issue(bb, (uint32_t)bb);
+                    if (ufirst() < nunits_s)
+                        for (int bb = 0; bb < Tile::NB - 1; ++bb) tile_issue(bb, ufirst() + (uint32_t)bb * udir());
                 }
                 constexpr bool kPiped = kPipe && S;
                 StencilPipe<T, kPipe ? L : 1, VEC> pipe(plcg_dsm);
                 uint32_t lr0 = 0, lr1 = 0;   // the staged units' x neighbours (this unit, the next)
-                auto pipe_issue = [&](int stage, uint32_t j) -> uint32_t {   // the sweep's unit number j
+                auto pipe_issue = [&](int stage, uint32_t uu) -> uint32_t {   // unit uu, if it exists
                     uint32_t lr = 0;
                     if constexpr (kPiped) {
-                        const uint32_t g = (ufirst + j * udir) * usw + (uint32_t)tid * VEC;
-                        const bool in = j < ucnt && g < nn;
+                        const uint32_t g = uu * usw + (uint32_t)tid * VEC;
+                        const bool in = uu < nunits_s && g < nn;
                         const uint32_t gs = in ? g : 0u;
-                        if (j < ucnt) {
-                            lr = pipe.issue_z(stage, st, C.zl_cur, gs, in);
+                        if (uu < nunits_s) {
+                            lr = pipe.issue_z(stage, st, C.zl_cur, gs, in, PAD ? a.nxr : 0);
                             cp_async_cg16(pipe.slot(stage, 5), C.zl_prev + gs, in);
 #pragma unroll
                             for (int k = 0; k < L; ++k) {
@@ -2141,14 +2206,15 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
                     }
                     return lr;
                 };
-                lr0 = pipe_issue(0, 0);
-                lr1 = pipe_issue(1, 1);
+                int ps = 0;                  // this unit's stage
+                lr0 = pipe_issue(0, ufirst());
+                lr1 = pipe_issue(1, ufirst() + udir());
                 typename CsrStage<CT>::Rows rp_next{0, 0};   // the warp's next unit's row pointers
                 if constexpr (kStage) {
-                    const uint32_t w0 = ufirst * usw + (uint32_t)(tid & ~31);
-                    if (a.stage && ucnt > 0 && w0 < nn) rp_next = CsrStage<CT>::rows_load(csr, w0, min(w0 + 32u, nn));
+                    const uint32_t w0 = ufirst() * usw + (uint32_t)(tid & ~31);
+                    if (a.stage && w0 < nn) rp_next = CsrStage<CT>::rows_load(csr, w0, min(w0 + 32u, nn));
                 }
-                for (uint32_t j = 0, u = ufirst; j < ucnt; ++j, u += udir) {
+                for (uint32_t u = ufirst(); u < nunits_s; u += udir()) {
                     uint32_t g0[RPT];
                     bool ok[RPT];
 #pragma unroll
@@ -2162,8 +2228,8 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
                         const uint32_t w0 = u * usw + (uint32_t)(tid & ~31);
                         if (a.stage && w0 < nn) {
                             const typename CsrStage<CT>::Rows rp = rp_next;
-                            const uint32_t wn = w0 + udir * usw;
-                            if (j + 1 < ucnt && wn < nn)
+                            const uint32_t wn = w0 + udir() * usw;
+                            if (u + udir() < nunits_s && wn < nn)
                                 rp_next = CsrStage<CT>::rows_load(csr, wn, min(wn + 32u, nn));
                             int64_t e0, e1;
                             CsrStage<CT>::rows_bounds(rp, &e0, &e1, &rs, &re);
@@ -2173,7 +2239,7 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
                     T bw[13];   // the tiled unit's backward coefficients (row g0[0])
                     if constexpr (kTile) {    // the copies NB - 1 units ahead; this unit's tile
                         stg = (stg_q >> tb) & 1u;
-                        tile_issue((tb + Tile::NB - 1) % Tile::NB, j + (uint32_t)(Tile::NB - 1));
+                        tile_issue((tb + Tile::NB - 1) % Tile::NB, u + (uint32_t)(Tile::NB - 1) * udir());
                         if (stg && ok[0]) tile.backward(g0[0], bw);
                         if (stg) tile.wait(tb, a.poll_limit, &a.out->abort);
                     }
@@ -2187,18 +2253,17 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
                         for (int v = 0; v < VEC; ++v) zp[r][v] = T(0);
                         dg[r] = T(1);
                         if constexpr (kPiped) {
-                            const int stage = (int)(j & 1u);
                             cp_async_wait<1>();
-                            pipe.parts(stage, st.dim == 3, lr0, c[r], nb[r]);
-                            pipe.get(stage, 5, zp[r]);
+                            pipe.parts(ps, st.dim == 3, lr0, c[r], nb[r]);
+                            pipe.get(ps, 5, zp[r]);
 #pragma unroll
                             for (int k = 0; k < L; ++k) {
-                                pipe.get(stage, 6 + k, cur[r][k]);
-                                pipe.get(stage, 6 + L + k, pk[r][k]);
+                                pipe.get(ps, 6 + k, cur[r][k]);
+                                pipe.get(ps, 6 + L + k, pk[r][k]);
                             }
                             if (k6 != 3) {
-                                pipe.get(stage, 6 + 2 * L, pv[r]);
-                                pipe.get(stage, 7 + 2 * L, xv[r]);
+                                pipe.get(ps, 6 + 2 * L, pv[r]);
+                                pipe.get(ps, 7 + 2 * L, xv[r]);
                             }
                             continue;
                         }
@@ -2321,6 +2386,11 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
                                     }
                             }
                         }
+                        if constexpr (PAD) {
+                            const int cnt = kPiped ? (int)(lr0 >> 2) : pad_rows<PAD, VEC>(a, g0[r]).cnt;
+#pragma unroll
+                            for (int v = 0; v < VEC; ++v) un[v] = v < cnt ? un[v] : T(0);
+                        }
                         // K6: p and the iterate (Algorithm 1, K6)
                         if (k6 == 1) {
 #pragma unroll
@@ -2378,7 +2448,8 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
                     }
                     if constexpr (kPiped) {   // this unit's slots are free
                         lr0 = lr1;
-                        lr1 = pipe_issue((int)(j & 1u), j + 2);
+                        lr1 = pipe_issue(ps, u + 2 * udir());
+                        ps ^= 1;
                     }
                     tb = (tb + 1) % Tile::NB;
                 }
@@ -2388,11 +2459,14 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
             // fetched anew in every launch, and a second loop's cost more than
             // the test)
             constexpr bool kSplit = std::is_same<Grp, BlockGroup<T>>::value || VEC > 1 || kTile;
-            if (!steady) sweep(std::false_type{}, std::integral_constant<int, 0>{});
-            else if constexpr (!kPair) sweep(std::true_type{}, std::integral_constant<int, 4>{});
-            else if constexpr (!kSplit) sweep(std::true_type{}, std::integral_constant<int, 0>{});
-            else if (C.k6 == 2) sweep(std::true_type{}, std::integral_constant<int, 2>{});
-            else sweep(std::true_type{}, std::integral_constant<int, 3>{});
+            if (steady) {
+                if constexpr (!kPair) sweep(std::true_type{}, std::integral_constant<int, 4>{});
+                else if constexpr (!kSplit) sweep(std::true_type{}, std::integral_constant<int, 0>{});
+                else if (C.k6 == 2) sweep(std::true_type{}, std::integral_constant<int, 2>{});
+                else sweep(std::true_type{}, std::integral_constant<int, 3>{});
+            } else {
+                sweep(std::false_type{}, std::integral_constant<int, 0>{});
+            }
             double acc[2 * L + 1];
 #pragma unroll
             for (int q = 0; q <= 2 * L; ++q) {
@@ -2521,7 +2595,7 @@ __device__ void cg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
     } while (0)
 
     for (;;) {
-        residual_sweep<T, VEC, OP, Grp, CT>(a, s, grp);
+        residual_sweep<T, VEC, OP, Grp, CT>(a, a.st, s, grp);
         grp.put_norms(a, s);
         spmvs++;
         CG_SYNC();
@@ -2836,20 +2910,24 @@ finish:
 // ------------------------------------------------------------------------
 // CTAs per SM the register budget is sized for: two for the sweeps whose
 // operands are copied ahead (their slots' shared memory), three for the other
-// FP32 sweeps with l <= 2, two otherwise; the 27-point tiles' buffers (about
+// FP32 sweeps with l <= 2 and the FP64 p(1)-CG stencil sweep with scaled bases
+// and two rows per thread (3D 256^3 161.7 -> 138.5 ms at 85 registers with 72
+// bytes of spills, against 128 registers at two CTAs per SM), two otherwise; the 27-point tiles' buffers (about
 // 47 KB each) leave room for one CTA per SM with four of them (two with two).
-template <typename T, int L, int OP, bool SC = false, int VEC = 1>
-constexpr int kPlcgMinBlocks = (sizeof(T) == 4 && L <= 2 && !op_is_var27(OP) && !pipe_used(OP, VEC, L)) ? 3 : 2;
+template <typename T, int L, int OP, bool SC = false, int VEC = 1, bool PIPE = false>
+constexpr int kPlcgMinBlocks = (sizeof(T) == 4 && L <= 2 && !op_is_var27(OP) && !PIPE)    ? 3
+                               : (SC && L == 1 && OP == kOpStencil && VEC == 2 && !PIPE) ? 3
+                                                                                         : 2;
 
 // CT: the stored type of the matrix values (T, or float under FP64 vectors:
 // the FP32-matrix path).
-template <typename T, int L, int VEC, int OP, bool SC = false, typename CT = T>
-__global__ void __launch_bounds__(kBlock, (kPlcgMinBlocks<T, L, OP, SC, VEC>))
+template <typename T, int L, int VEC, int OP, bool SC = false, typename CT = T, bool PIPE = false, bool PAD = false>
+__global__ void __launch_bounds__(kBlock, (kPlcgMinBlocks<T, L, OP, SC, VEC, PIPE>))
 plcg_kernel(SolveArgs<T> a)
 {
     __shared__ Smem<T> s;
     GridGroup<T> grp;
-    plcg_body<T, L, VEC, OP, GridGroup<T>, 1, SC, CT>(a, s, grp);
+    plcg_body<T, L, VEC, OP, GridGroup<T>, 1, SC, CT, false, PIPE, PAD>(a, s, grp);
 }
 
 template <typename T, int VEC, int OP, typename CT = T>
