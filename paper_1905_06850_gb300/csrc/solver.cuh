@@ -258,6 +258,88 @@ __device__ __forceinline__ void warp_partials_sum(const double *part, int count,
     __syncwarp();
 }
 
+// Partials kept dot by dot, part[q * count + c] (a warp's loads are whole lines):
+// one warp's sums as above, four loads of each dot in flight; and the whole
+// CTA's, a thread or two per partial, in dst[q] for the first warp.
+template <int ND, int Q0>
+__device__ __forceinline__ void warp_columns_sum(const double *part, int count, double *dst)
+{
+    constexpr int NA = ND - Q0;
+    constexpr int P = NA <= 1 ? 0 : NA <= 2 ? 1 : NA <= 4 ? 2 : NA <= 8 ? 3 : NA <= 16 ? 4 : 5;
+    const int lane = threadIdx.x & 31;
+    double v[NA];
+#pragma unroll
+    for (int q = 0; q < NA; ++q) v[q] = 0.0;
+    int c = lane;
+    for (; c + 96 < count; c += 128) {
+        double w[4][NA];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int q = 0; q < NA; ++q) w[j][q] = __ldcg(part + (size_t)(Q0 + q) * count + c + 32 * j);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int q = 0; q < NA; ++q) v[q] += w[j][q];
+    }
+    for (; c < count; c += 32) {
+#pragma unroll
+        for (int q = 0; q < NA; ++q) v[q] += __ldcg(part + (size_t)(Q0 + q) * count + c);
+    }
+    const double t = warp_reduce_scatter<NA>(v, lane);
+    if ((lane & ((32 >> P) - 1)) == 0) {
+        const int q = lane >> (5 - P);
+        if (q < NA) dst[Q0 + q] = t;
+    }
+    if (lane < Q0) dst[lane] = 0.0;
+    __syncwarp();
+}
+
+template <int ND, int Q0>
+__device__ __forceinline__ void block_columns_sum(const double *part, int count, double *s_red, double *dst)
+{
+    constexpr int NA = ND - Q0;
+    constexpr int P = NA <= 1 ? 0 : NA <= 2 ? 1 : NA <= 4 ? 2 : NA <= 8 ? 3 : NA <= 16 ? 4 : 5;
+    constexpr int W = kBlock / 32;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    double v[NA], v2[NA];
+    const int c0 = threadIdx.x, c1 = c0 + kBlock;
+#pragma unroll
+    for (int q = 0; q < NA; ++q) {
+        const double *col = part + (size_t)(Q0 + q) * count;
+        v[q] = c0 < count ? __ldcg(col + c0) : 0.0;
+        v2[q] = c1 < count ? __ldcg(col + c1) : 0.0;
+    }
+    if (warp * 32 + kBlock < count) {
+#pragma unroll
+        for (int q = 0; q < NA; ++q) v[q] += v2[q];
+        for (int c = c1 + kBlock; c < count; c += kBlock) {
+#pragma unroll
+            for (int q = 0; q < NA; ++q) v[q] += __ldcg(part + (size_t)(Q0 + q) * count + c);
+        }
+    }
+    const double t = warp * 32 < count ? warp_reduce_scatter<NA>(v, lane) : 0.0;
+    if ((lane & ((32 >> P) - 1)) == 0) {
+        const int q = lane >> (5 - P);
+        if (q < NA) s_red[warp * NA + q] = t;
+    }
+    __syncthreads();
+    if (warp == 0) {
+        if (lane < NA) {
+            double w8[W];
+#pragma unroll
+            for (int w = 0; w < W; ++w) w8[w] = s_red[w * NA + lane];
+#pragma unroll
+            for (int h = W / 2; h >= 1; h >>= 1)
+#pragma unroll
+                for (int w = 0; w < h; ++w) w8[w] += w8[w + h];
+            dst[Q0 + lane] = w8[0];
+        }
+        if (lane < Q0) dst[lane] = 0.0;
+        __syncwarp();
+    }
+}
+
 // The dots of the partial ring a scalar step needs: all 2l+1 positions with
 // the 2l+1-dot variant, positions l .. 2l with the l+1 dots of Sec. 2.2.
 template <int ND>
@@ -1133,17 +1215,18 @@ struct GridGroup {
     __device__ __forceinline__ void put_dots(const SolveArgs<T> &a, Smem<T> &s, int slot, int nd)
     {
         if ((int)threadIdx.x < nd)
-            a.part[((size_t)slot * gridDim.x + blockIdx.x) * kMaxDots + threadIdx.x] = s.out[threadIdx.x];
+            a.part[((size_t)slot * kMaxDots + threadIdx.x) * gridDim.x + blockIdx.x] = s.out[threadIdx.x];
     }
     // sum over CTAs of ring slot `slot` into dst[0..ND)
     template <int ND>
     __device__ __forceinline__ void get_dots(const SolveArgs<T> &a, Smem<T> &s, int slot, double *dst)
     {
-        // warp 0 sums (few FP64 instructions: GB300's FP64 units are narrow),
-        // the CTA barrier publishes the result
-        if (threadIdx.x < 32)
-            warp_partials_sum<ND>(a.part + (size_t)slot * gridDim.x * kMaxDots, (int)gridDim.x, kMaxDots, dst);
+        block_columns_sum<ND, 0>(column(a, slot), (int)gridDim.x, s.red, dst);
         __syncthreads();
+    }
+    __device__ __forceinline__ const double *column(const SolveArgs<T> &a, int slot) const
+    {
+        return a.part + (size_t)slot * kMaxDots * gridDim.x;
     }
     // one warp sums ring slot `slot` over the CTAs into dst (every CTA's warp
     // adds in the same order, so all CTAs get the same bits)
@@ -1151,8 +1234,15 @@ struct GridGroup {
     __device__ __forceinline__ void get_dots_warp(const SolveArgs<T> &a, Smem<T> &, int slot,
                                                   double *dst)
     {
-        warp_dots_sum<ND>(a.part + (size_t)slot * gridDim.x * kMaxDots, (int)gridDim.x, kMaxDots,
-                          a.dots_2l1 != 0, dst);
+        if (a.dots_2l1) warp_columns_sum<ND, 0>(column(a, slot), (int)gridDim.x, dst);
+        else warp_columns_sum<ND, (ND - 1) / 2>(column(a, slot), (int)gridDim.x, dst);
+    }
+    // the same by all threads of the CTA; dst is warp 0's
+    template <int ND>
+    __device__ __forceinline__ void get_dots_all(const SolveArgs<T> &a, Smem<T> &s, int slot, double *dst)
+    {
+        if (a.dots_2l1) block_columns_sum<ND, 0>(column(a, slot), (int)gridDim.x, s.red, dst);
+        else block_columns_sum<ND, (ND - 1) / 2>(column(a, slot), (int)gridDim.x, s.red, dst);
     }
     __device__ __forceinline__ void put_norms(const SolveArgs<T> &a, Smem<T> &s)
     {
@@ -2489,9 +2579,12 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
             grp.put_dots(a, s, (int)(i % (L + 1)), 2 * L + 1);
             PLCG_SYNC();
             if (!la) {   // MPI_Wait(req(i+1-l)) and the scalar step, serially (warp 0)
+                if constexpr (kGrid)
+                    if (i + 1 >= L) grp.template get_dots_all<2 * L + 1>(a, s, (int)((i + 1 - L) % (L + 1)), s.raw);
                 if (tid < 32) {
-                    if (i + 1 >= L)
-                        grp.template get_dots_warp<2 * L + 1>(a, s, (int)((i + 1 - L) % (L + 1)), s.raw);
+                    if constexpr (!kGrid)
+                        if (i + 1 >= L)
+                            grp.template get_dots_warp<2 * L + 1>(a, s, (int)((i + 1 - L) % (L + 1)), s.raw);
                     if (tid == 0)
                         scalar_step<T, L, kOolScalar, SC, kPair>(s, s.cfb[(i + 1) & 1], s.raw, a, (int)(i + 1), rn, tau,
                                                       budget, kc, kn);
