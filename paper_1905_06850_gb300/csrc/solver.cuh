@@ -21,6 +21,7 @@
 
 #include <type_traits>
 
+#include "fastroot.h"
 #include "fxsum.h"
 #include "plcg_internal.h"
 
@@ -59,10 +60,13 @@ __device__ __forceinline__ unsigned long long global_timer_ns()
 // e is passed when *bar reaches e * gridDim.x.  Returns false when the poll
 // bound ran out (the CTA then sets the abort flag) or another CTA aborted;
 // the caller must then leave the kernel.  force_timeout adds one phantom
-// arrival to the target so that the wait runs out (test hook).
+// arrival to the target so that the wait runs out (test hook).  A CTA whose
+// own copies did not land (s_quit, in shared memory) does not arrive, so nobody
+// passes: the abort flag, in global memory, is looked at in the polls only (a
+// look after each wait is a round trip to the L2 more, 0.3 us).
 __device__ __forceinline__ bool group_barrier(unsigned *bar, unsigned &epoch, unsigned members,
                                               unsigned long long limit, int force,
-                                              int *abort_flag, int *s_ok)
+                                              int *abort_flag, int *s_ok, const int *s_quit)
 {
     // bar.sync orders the CTA's writes before thread 0's release-add (release
     // is cumulative over what happened before it); the acquire-load that sees
@@ -71,17 +75,16 @@ __device__ __forceinline__ bool group_barrier(unsigned *bar, unsigned &epoch, un
     if (threadIdx.x == 0) {
         epoch += 1u;
         const unsigned target = epoch * members + (force ? 1u : 0u);
-        red_release_add_u32(bar, 1u);
-        int ok = 1;
+        int ok = s_quit && ld_volatile(s_quit) ? 0 : 1;
         unsigned long long polls = 0;
-        while ((int)(ld_acquire_u32(bar) - target) < 0) {
+        if (ok) red_release_add_u32(bar, 1u);
+        while (ok && (int)(ld_acquire_u32(bar) - target) < 0) {
             if ((++polls & 31) == 0) {
                 if (ld_volatile(abort_flag)) { ok = 0; break; }
                 if (polls > limit) { atomicExch(abort_flag, 1); ok = 0; break; }
                 __nanosleep(32);
             }
         }
-        if (ok && ld_volatile(abort_flag)) ok = 0;
         *s_ok = ok;
     }
     __syncthreads();
@@ -90,9 +93,9 @@ __device__ __forceinline__ bool group_barrier(unsigned *bar, unsigned &epoch, un
 
 __device__ __forceinline__ bool grid_barrier(unsigned *bar, unsigned &epoch,
                                              unsigned long long limit, int force,
-                                             int *abort_flag, int *s_ok)
+                                             int *abort_flag, int *s_ok, const int *s_quit)
 {
-    return group_barrier(bar, epoch, gridDim.x, limit, force, abort_flag, s_ok);
+    return group_barrier(bar, epoch, gridDim.x, limit, force, abort_flag, s_ok, s_quit);
 }
 
 // ------------------------------------------------------------------------
@@ -811,11 +814,12 @@ struct Var27Tile {
     }
     // Wait for the copies issue() started (bounded: on timeout the abort flag
     // is raised and the wait repeated once, so no copy is left in flight).
-    __device__ __forceinline__ void wait(int buf, unsigned long long limit, int *abort_flag)
+    __device__ __forceinline__ void wait(int buf, unsigned long long limit, int *abort_flag, int *s_quit)
     {
         const uint32_t ph = (parity >> buf) & 1u;
         if (!mbar_wait(bar + buf, ph, limit)) {
             atomicExch(abort_flag, 1);
+            *(volatile int *)s_quit = 1;
             mbar_wait(bar + buf, ph, limit);
         }
         parity ^= 1u << buf;
@@ -1032,7 +1036,7 @@ struct CsrStage {
     // Returns false (read global memory) when the range exceeds the warp's
     // buffer; *e0s is the global position of the first staged entry.
     __device__ __forceinline__ bool stage_range(const CsrDesc &csr, int64_t e0, int64_t e1, int64_t *e0s,
-                                                unsigned long long limit, int *abort_flag)
+                                                unsigned long long limit, int *abort_flag, int *s_quit)
     {
         *e0s = e0 & ~int64_t(3);
         const int64_t cnt = ((e1 + 3) & ~int64_t(3)) - *e0s;
@@ -1049,6 +1053,7 @@ struct CsrStage {
             }
             if (!mbar_wait(bar, parity, limit)) {
                 atomicExch(abort_flag, 1);          // the solve ends at the next barrier
+                *(volatile int *)s_quit = 1;
                 mbar_wait(bar, parity, limit);      // the copy in flight lands first
             }
             parity ^= 1u;
@@ -1179,6 +1184,7 @@ struct Smem {
     long long stg_e0;                // CSR staging: global position of the unit's first staged entry
     int stg_on;                      // CSR staging: this unit's entries are in shared memory
     int ok;
+    int quit;                        // whole grid: a bulk copy of this CTA did not land in time
 };
 
 template <typename T> struct Eps;
@@ -1209,7 +1215,7 @@ struct GridGroup {
     __device__ __forceinline__ bool leader() const { return blockIdx.x == 0; }
     __device__ __forceinline__ bool sync(const SolveArgs<T> &a, Smem<T> &s)
     {
-        return grid_barrier(a.bar, epoch, a.poll_limit, a.force_timeout, &a.out->abort, &s.ok);
+        return grid_barrier(a.bar, epoch, a.poll_limit, a.force_timeout, &a.out->abort, &s.ok, &s.quit);
     }
     // this CTA's reduced dots (s.out[0..nd)) into ring slot `slot`
     __device__ __forceinline__ void put_dots(const SolveArgs<T> &a, Smem<T> &s, int slot, int nd)
@@ -1412,7 +1418,7 @@ struct GangGroup {
     __device__ __forceinline__ bool leader() const { return rank == 0; }
     __device__ __forceinline__ bool sync(const SolveArgs<T> &, Smem<T> &s)
     {
-        return group_barrier(bar, epoch, (unsigned)G, limit, 0, abort_flag, &s.ok);
+        return group_barrier(bar, epoch, (unsigned)G, limit, 0, abort_flag, &s.ok, nullptr);
     }
     __device__ __forceinline__ void put_dots(const SolveArgs<T> &, Smem<T> &s, int slot, int nd)
     {
@@ -1463,6 +1469,7 @@ __device__ __forceinline__ void step_vectors(Coef<T> &cf, const SolveArgs<T> &a,
 {
     const int m = i - L;
     const bool rec = i >= L;
+    cf.ncopy = 0;
     cf.zl_cur = ring(a, L, i);
     cf.zl_prev = (i >= 1) ? ring(a, L, i - 1) : nullptr;
     cf.zl_new = ring(a, L, i + 1);
@@ -1542,17 +1549,19 @@ template <typename T, int L, int VEC, int OP, class Grp>
 constexpr bool kPairK6 = kPairIn<T, Grp> && OP == kOpStencil && !(L == 1 && sizeof(T) == 8) &&
                          (VEC > 1 || !std::is_same<Grp, GridGroup<T>>::value);
 
-template <typename T, int L, bool SC, bool PAIR>
+// vectors: false where step_vectors has already run for this i.  FAST: the
+// reciprocals of fastroot.h (fewer dependent FP64 instructions); the one-CTA and
+// gang groups keep the plain ones.
+template <typename T, int L, bool SC, bool PAIR, bool FAST>
 __device__ __forceinline__ void scalar_step_body(Smem<T> &s, Coef<T> &cf, const double *raw,
                                                  const SolveArgs<T> &a, int i, double rn,
-                                                 double tau, long long budget, T kc, T kn)
+                                                 double tau, long long budget, T kc, T kn, bool vectors)
 {
     cf.end = -1;
     cf.fmode = 0;
-    cf.ncopy = 0;
     cf.unit = 0;
     const int m = i - L;
-    step_vectors<T, L>(cf, a, i);
+    if (vectors) step_vectors<T, L>(cf, a, i);
     constexpr bool kScaled = SC && kScaledBases<T, L>;
     const bool scl = kScaled && kn != T(0);
     if (i < L) {
@@ -1611,7 +1620,7 @@ __device__ __forceinline__ void scalar_step_body(Smem<T> &s, Coef<T> &cf, const 
     const double graw = col[2 * L];
     double arg = graw;
     for (int k = lo; k <= c - 1; ++k) arg -= col[k - c + 2 * L] * col[k - c + 2 * L];
-    const double rg = rsqrt(arg);          // NaN or inf when arg <= 0: unused then
+    const double rg = FAST ? fast_rsqrt(arg) : rsqrt(arg);   // NaN or inf when arg <= 0: unused then
     const double gmm = g(m, m), igmm = ginv(m);
     const double gmc = col[m - c + 2 * L];
     const double dm1 = del(m - 1);        // delta_{m-1} (0 for m = 0)
@@ -1626,7 +1635,7 @@ __device__ __forceinline__ void scalar_step_body(Smem<T> &s, Coef<T> &cf, const 
     if (m >= 1) {
         lam = dm1 * s.ieta[(m - 1) & 1];
         em = gm - lam * dm1;
-        iem = 1.0 / em;
+        iem = FAST ? fast_rcp(em) : 1.0 / em;
         zm = -lam * s.zeta[(m - 1) & 1];
     }
     const double thr = 64.0 * Eps<T>::v * fabs(graw);
@@ -1764,12 +1773,12 @@ __device__ __forceinline__ void scalar_step_body(Smem<T> &s, Coef<T> &cf, const 
     }
 }
 
-template <typename T, int L, bool SC, bool PAIR>
+template <typename T, int L, bool SC, bool PAIR, bool FAST>
 __device__ __noinline__ void scalar_step_call(Smem<T> &s, Coef<T> &cf, const double *raw,
                                               const SolveArgs<T> &a, int i, double rn, double tau,
-                                              long long budget, T kc, T kn)
+                                              long long budget, T kc, T kn, bool vectors)
 {
-    scalar_step_body<T, L, SC, PAIR>(s, cf, raw, a, i, rn, tau, budget, kc, kn);
+    scalar_step_body<T, L, SC, PAIR, FAST>(s, cf, raw, a, i, rn, tau, budget, kc, kn, vectors);
 }
 
 // The scalar step inline, except in the FP32 whole-grid kernels: there the
@@ -1777,13 +1786,13 @@ __device__ __noinline__ void scalar_step_call(Smem<T> &s, Coef<T> &cf, const dou
 // changes its register allocation enough to cost ~15% at 256^3 (measured);
 // the out-of-line call costs ~0.3 us per iteration, which the FP64 and
 // one-CTA paths (latency-bound on small systems) keep.
-template <typename T, int L, bool OOL, bool SC, bool PAIR>
+template <typename T, int L, bool OOL, bool SC, bool PAIR, bool FAST>
 __device__ __forceinline__ void scalar_step(Smem<T> &s, Coef<T> &cf, const double *raw,
                                             const SolveArgs<T> &a, int i, double rn, double tau,
-                                            long long budget, T kc, T kn)
+                                            long long budget, T kc, T kn, bool vectors = true)
 {
-    if constexpr (OOL) scalar_step_call<T, L, SC, PAIR>(s, cf, raw, a, i, rn, tau, budget, kc, kn);
-    else scalar_step_body<T, L, SC, PAIR>(s, cf, raw, a, i, rn, tau, budget, kc, kn);
+    if constexpr (OOL) scalar_step_call<T, L, SC, PAIR, FAST>(s, cf, raw, a, i, rn, tau, budget, kc, kn, vectors);
+    else scalar_step_body<T, L, SC, PAIR, FAST>(s, cf, raw, a, i, rn, tau, budget, kc, kn, vectors);
 }
 
 // Per-thread accumulator of one dot product over the units a thread sweeps.
@@ -1944,6 +1953,9 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
     constexpr bool kF32 = (sizeof(T) == 4);
     constexpr bool kGrid = std::is_same<Grp, GridGroup<T>>::value;
     constexpr bool kOolScalar = kF32 && kGrid;
+    // the next step's vector pointers are set while the CTA waits at the barrier
+    constexpr bool kEarly = kGrid && L == 1;
+    constexpr bool kFast = kGrid || std::is_same<Grp, ClusterGroup<T>>::value;
     // FP64 p(1)-CG keeps its bases scaled (see scalar_step_body): two FP64
     // multiplies per row fewer in the FP64-bound sweep
     constexpr bool kScaled = SC && kScaledBases<T, L>;
@@ -2105,7 +2117,7 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
             const uint32_t u0 = (uint32_t)grp.unit0(), us = (uint32_t)grp.ustep();
             ulast = u0 < units ? u0 + (units - 1 - u0) / us * us : u0;
         }
-        if (tid == 0) scalar_step<T, L, kOolScalar, SC, kPair>(s, s.cfb[0], s.raw, a, 0, rn, tau, budget, kc, kn);
+        if (tid == 0) scalar_step<T, L, kOolScalar, SC, kPair, kFast>(s, s.cfb[0], s.raw, a, 0, rn, tau, budget, kc, kn);
         __syncthreads();
         for (long long i = 0;; ++i) {
             const Coef<T> &cf = s.cfb[i & 1];
@@ -2180,7 +2192,7 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
                 if (i + 1 >= L)
                     grp.template get_dots_warp<2 * L + 1>(a, s, (int)((i + 1 - L) % (L + 1)), s.raw2);
                 if ((tid & 31) == 0)
-                    scalar_step<T, L, kOolScalar, SC, kPair>(s, s.cfb[(i + 1) & 1], s.raw2, a, (int)(i + 1), rn, tau, budget,
+                    scalar_step<T, L, kOolScalar, SC, kPair, kFast>(s, s.cfb[(i + 1) & 1], s.raw2, a, (int)(i + 1), rn, tau, budget,
                                                   kc, kn);
                 __syncwarp();
             }
@@ -2323,7 +2335,7 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
                                 rp_next = CsrStage<CT>::rows_load(csr, wn, min(wn + 32u, nn));
                             int64_t e0, e1;
                             CsrStage<CT>::rows_bounds(rp, &e0, &e1, &rs, &re);
-                            stg = stage.stage_range(csr, e0, e1, &e0s, a.poll_limit, &a.out->abort);
+                            stg = stage.stage_range(csr, e0, e1, &e0s, a.poll_limit, &a.out->abort, &s.quit);
                         }
                     }
                     T bw[13];   // the tiled unit's backward coefficients (row g0[0])
@@ -2331,7 +2343,7 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
                         stg = (stg_q >> tb) & 1u;
                         tile_issue((tb + Tile::NB - 1) % Tile::NB, u + (uint32_t)(Tile::NB - 1) * udir());
                         if (stg && ok[0]) tile.backward(g0[0], bw);
-                        if (stg) tile.wait(tb, a.poll_limit, &a.out->abort);
+                        if (stg) tile.wait(tb, a.poll_limit, &a.out->abort, &s.quit);
                     }
                     // -- loads
                     T c[RPT][VEC], nb[RPT][VEC], zp[RPT][VEC], cur[RPT][L][VEC], pk[RPT][L][VEC];
@@ -2577,6 +2589,8 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
                 if (tid < L) s.out[tid] = 0.0;
             }
             grp.put_dots(a, s, (int)(i % (L + 1)), 2 * L + 1);
+            if constexpr (kEarly)
+                if (tid == kBlock - 1) step_vectors<T, L>(s.cfb[(i + 1) & 1], a, (int)(i + 1));
             PLCG_SYNC();
             if (!la) {   // MPI_Wait(req(i+1-l)) and the scalar step, serially (warp 0)
                 if constexpr (kGrid)
@@ -2586,8 +2600,8 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
                         if (i + 1 >= L)
                             grp.template get_dots_warp<2 * L + 1>(a, s, (int)((i + 1 - L) % (L + 1)), s.raw);
                     if (tid == 0)
-                        scalar_step<T, L, kOolScalar, SC, kPair>(s, s.cfb[(i + 1) & 1], s.raw, a, (int)(i + 1), rn, tau,
-                                                      budget, kc, kn);
+                        scalar_step<T, L, kOolScalar, SC, kPair, kFast>(s, s.cfb[(i + 1) & 1], s.raw, a, (int)(i + 1),
+                                                                        rn, tau, budget, kc, kn, !kEarly);
                 }
                 __syncthreads();
             }
@@ -2827,7 +2841,7 @@ __device__ void cg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
                     const uint32_t g = u * usw + (uint32_t)tid;
                     T bw[13];
                     if (stg && g < nn) tile.backward(g, bw);
-                    if (stg) tile.wait(tb, a.poll_limit, &a.out->abort);
+                    if (stg) tile.wait(tb, a.poll_limit, &a.out->abort, &s.quit);
                     if (g < nn) {
                         T c[VEC], w[VEC];
                         T mi = T(1);   // Jacobi: 1 / a_gg
@@ -2869,7 +2883,7 @@ __device__ void cg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
                                 rp_next = CsrStage<CT>::rows_load(csr, wn, min(wn + 32u, nn));
                             int64_t e0, e1;
                             CsrStage<CT>::rows_bounds(rp, &e0, &e1, &rs, &re);
-                            stg = stage.stage_range(csr, e0, e1, &e0s, a.poll_limit, &a.out->abort);
+                            stg = stage.stage_range(csr, e0, e1, &e0s, a.poll_limit, &a.out->abort, &s.quit);
                         }
                     }
 #pragma unroll
@@ -3020,6 +3034,7 @@ plcg_kernel(SolveArgs<T> a)
 {
     __shared__ Smem<T> s;
     GridGroup<T> grp;
+    if (threadIdx.x == 0) s.quit = 0;
     plcg_body<T, L, VEC, OP, GridGroup<T>, 1, SC, CT, false, PIPE, PAD>(a, s, grp);
 }
 
@@ -3028,6 +3043,7 @@ __global__ void __launch_bounds__(kBlock, 3) cg_kernel(SolveArgs<T> a)
 {
     __shared__ Smem<T> s;
     GridGroup<T> grp;
+    if (threadIdx.x == 0) s.quit = 0;
     cg_body<T, VEC, OP, GridGroup<T>, 1, CT>(a, s, grp);
 }
 
