@@ -2665,6 +2665,14 @@ __device__ void cg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
     // FP64 FMA at every stencil point or matrix entry (one pass more, 7 of 18
     // FP64 instructions per row fewer on the 7-point stencil)
     constexpr bool kSepP = kTileCG || (sizeof(T) == 8 && std::is_same<Grp, GridGroup<T>>::value && RPT == 1);
+    // There x takes step k - 1 in the p sweep of step k, where p_{k-1} passes by
+    // anyway (ten vector passes an iteration instead of eleven, the same
+    // operations), and the two vector sweeps load two units' rows before they
+    // store the first's: with one unit's 16-byte loads a thread the sweeps waited
+    // for memory.  3D 160^3 100.1 -> 90.2 us per iteration (96.0 with one unit at
+    // a time), 256^3 378 -> 323; where a CTA has one unit nothing changes.  Not
+    // CSR (FP64 128^3 214.8 -> 224.5).
+    constexpr bool kLateX = kSepP && !kTileCG && !op_is_csr(OP);
     using Tile = Var27Tile<T, 0, kV27StageBwdCg>;
     Tile tile(plcg_dsm);
     if constexpr (kSepP) {
@@ -2775,7 +2783,8 @@ __device__ void cg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
         }
         long long k = 0;
         int end;
-        double beta = 0.0;
+        double beta = 0.0, alpha = 0.0;
+        bool owed = false;   // kLateX: x lacks alpha p
         for (;;) {
             if (!isfinite(rr)) { end = kSegNonfinite; break; }
             if (sqrt(rr) < tau) { end = kSegConverged; break; }
@@ -2786,7 +2795,45 @@ __device__ void cg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
             DotAcc<T, VEC> d1;
             int since_flush = 0;
             const int64_t nunits_s = (n + USWEEP - 1) / USWEEP;
-            if constexpr (kSepP) {
+            const uint32_t us = (uint32_t)grp.ustep();
+            if constexpr (kLateX) {
+                // p_k in place, x_k
+                auto rows = [&](uint32_t u, auto count) {
+                    constexpr int R = decltype(count)::value;
+                    T pv[R][VEC], zv[R][VEC], xv[R][VEC];
+                    uint32_t g0[R];
+                    bool in[R];
+#pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        g0[r] = (u + (uint32_t)r * us) * (uint32_t)UNIT + (uint32_t)tid * VEC;
+                        in[r] = g0[r] < nn;
+                        if (!in[r]) continue;
+                        vld<T, VEC>(rc + g0[r], zv[r]);
+                        if (k > 0) {
+                            vld<T, VEC>(pn + g0[r], pv[r]);
+                            vld<T, VEC>(xi + g0[r], xv[r]);
+                        }
+                    }
+#pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        if (!in[r]) continue;
+                        if (k > 0) {
+#pragma unroll
+                            for (int v = 0; v < VEC; ++v) {
+                                xv[r][v] = fma((T)alpha, pv[r][v], xv[r][v]);
+                                zv[r][v] = fma((T)beta, pv[r][v], zv[r][v]);
+                            }
+                            vst<T, VEC>(xi + g0[r], xv[r]);
+                        }
+                        vst<T, VEC>(pn + g0[r], zv[r]);
+                    }
+                };
+                uint32_t u = (uint32_t)grp.unit0();
+                for (; u + us < (uint32_t)nunits; u += 2 * us) rows(u, std::integral_constant<int, 2>{});
+                if (u < (uint32_t)nunits) rows(u, std::integral_constant<int, 1>{});
+                owed = false;
+                CG_SYNC();
+            } else if constexpr (kSepP) {
                 // p_k in place
                 for (int64_t u = grp.unit0(); u < nunits; u += grp.ustep()) {
                     const int64_t g0 = u * UNIT + (int64_t)tid * VEC;
@@ -2929,12 +2976,50 @@ __device__ void cg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
             grp.template get_dots<1>(a, s, 0, s.raw);
             const double pq = s.raw[0];
             if (!(pq > 0.0)) { end = isfinite(pq) ? kSegBreakdown : kSegNonfinite; break; }
-            const double alpha = rr / pq;
+            alpha = rr / pq;
+            owed = kLateX;
             const T al = (T)alpha;
             // ---- x += alpha p; r -= alpha q; (r, r)
             DotAcc<T, VEC> d2;
             since_flush = 0;
-            for (uint32_t u = (uint32_t)grp.unit0(); u < (uint32_t)nunits_s; u += (uint32_t)grp.ustep()) {
+            if constexpr (kLateX) {
+                auto rows = [&](uint32_t u, auto count) {
+                    constexpr int R = decltype(count)::value;
+                    T qv[R][VEC], rv[R][VEC], dv[R][VEC];
+                    uint32_t g0[R];
+                    bool in[R];
+#pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        g0[r] = (u + (uint32_t)r * us) * (uint32_t)UNIT + (uint32_t)tid * VEC;
+                        in[r] = g0[r] < nn;
+                        if (!in[r]) continue;
+                        vld<T, VEC>(q + g0[r], qv[r]);
+                        vld<T, VEC>(rc + g0[r], rv[r]);
+                        if constexpr (op_is_jacobi(OP)) {
+                            CT dc[VEC];
+                            vldg<CT, VEC>(static_cast<const CT *>(csr.diag) + g0[r], dc);
+#pragma unroll
+                            for (int v = 0; v < VEC; ++v) dv[r][v] = coef_cast<T>(dc[v]);
+                        }
+                    }
+#pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        if (!in[r]) continue;
+#pragma unroll
+                        for (int v = 0; v < VEC; ++v) {
+                            rv[r][v] = fma(-al, qv[r][v], rv[r][v]);
+                            if constexpr (op_is_jacobi(OP)) dv[r][v] *= rv[r][v];   // rho = (r, z) = sum a_gg z_g^2
+                        }
+                        vst<T, VEC>(rc + g0[r], rv[r]);
+                        if constexpr (op_is_jacobi(OP)) d2.add(dv[r], rv[r]);
+                        else d2.add(rv[r], rv[r]);
+                    }
+                };
+                uint32_t u = (uint32_t)grp.unit0();
+                for (; u + us < (uint32_t)nunits; u += 2 * us) rows(u, std::integral_constant<int, 2>{});
+                if (u < (uint32_t)nunits) rows(u, std::integral_constant<int, 1>{});
+            }
+            for (uint32_t u = (uint32_t)grp.unit0(); !kLateX && u < (uint32_t)nunits_s; u += us) {
                 T pv[RPT][VEC], qv[RPT][VEC], xv[RPT][VEC], rv[RPT][VEC], dv[RPT][VEC];
                 uint32_t g0[RPT];
 #pragma unroll
@@ -2991,6 +3076,18 @@ __device__ void cg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
         last_end = end;
         segments++;
         recres = sqrt(rr);
+        if (kLateX && owed) {
+            for (int64_t u = grp.unit0(); u < nunits; u += grp.ustep()) {
+                const int64_t g0 = u * UNIT + (int64_t)tid * VEC;
+                if (g0 >= n) continue;
+                T pv[VEC], xv[VEC];
+                vld<T, VEC>(pr[0] + g0, pv);
+                vld<T, VEC>(xi + g0, xv);
+#pragma unroll
+                for (int v = 0; v < VEC; ++v) xv[v] = fma((T)alpha, pv[v], xv[v]);
+                vst<T, VEC>(xi + g0, xv);
+            }
+        }
         if (end == kSegNonfinite) { status = kStNonfinite; goto finish; }
         if constexpr (kF32) {   // x += d
             for (int64_t u = grp.unit0(); u < nunits; u += grp.ustep()) {
