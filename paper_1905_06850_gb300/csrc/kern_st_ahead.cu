@@ -1,4 +1,4 @@
-// kern_st_ahead.cu -- instantiations of the persistent p(l)-CG solvers for large
+// kern_st_ahead.cu -- instantiations of the persistent solvers for large
 // stencil systems: sweeps whose operands are copied a unit ahead, and systems
 // whose lines are not whole 16-byte vectors, held at a padded pitch (FP64 with
 // scaled bases).
@@ -23,10 +23,11 @@ const void *kptr_st_ahead(bool f32, int l)
     }
 }
 
-const void *kptr_st_pad(bool f32, int l)
+const void *kptr_st_pad(bool f32, int l)   // l = 0: classic CG
 {
     if (f32) {
         switch (l) {
+        case 0: return reinterpret_cast<const void *>(&cg_kernel<float, 4, kOpStencil, float, true>);
         case 1: return reinterpret_cast<const void *>(&plcg_kernel<float, 1, 4, kOpStencil, false, float, true, true>);
         case 2: return reinterpret_cast<const void *>(&plcg_kernel<float, 2, 4, kOpStencil, false, float, true, true>);
         case 3: return reinterpret_cast<const void *>(&plcg_kernel<float, 3, 4, kOpStencil, false, float, false, true>);
@@ -34,6 +35,7 @@ const void *kptr_st_pad(bool f32, int l)
         }
     }
     switch (l) {
+    case 0: return reinterpret_cast<const void *>(&cg_kernel<double, 2, kOpStencil, double, true>);
     case 1: return reinterpret_cast<const void *>(&plcg_kernel<double, 1, 2, kOpStencil, true, double, true, true>);
     case 2: return reinterpret_cast<const void *>(&plcg_kernel<double, 2, 2, kOpStencil, true, double, true, true>);
     case 3: return reinterpret_cast<const void *>(&plcg_kernel<double, 3, 2, kOpStencil, true, double, false, true>);

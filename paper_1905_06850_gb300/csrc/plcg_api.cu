@@ -74,6 +74,8 @@ constexpr int64_t kVec1Rows = 16384;
 // 128^3; FP32 p(1) 80^3 15.1 and 13.5, 112^3 17.8 and 17.6, 176^3 47.6 and 40.8,
 // but between (its vectors fit the L2, and the third CTA hides more of the
 // latency) 136 x 125 x 118 15.3 and 15.6, 128^3 20.0 and 20.4, 144^3 25.3 and 25.6.
+constexpr int64_t kPadRows = 3 << 14;   // rows from which lines are padded (see build_solve)
+
 static bool copies_ahead(bool f32, int l, int64_t n)
 {
     // (the 2 l + 1 dots' loop does not copy ahead)
@@ -529,17 +531,20 @@ static plcg_status build_solve(const plcg_matrix *A, const double *b, double *x,
     // one row per thread.  3D 131^3 and 161^3, us per iteration, FP32 p(1)-CG
     // 30 -> 22 and 59 -> 34, p(2) 34 -> 22 and 68 -> 38, p(3) 53 -> 29 and 95 ->
     // 51; FP64 66 -> 51 and 113 -> 84, 75 -> 61 and 134 -> 104, 87 -> 74 and 155
-    // -> 126; 69^3 FP32 15.3 -> 13.4, 17.1 -> 13.8, 16.1 -> 16.2.
+    // -> 126; 69^3 FP32 15.3 -> 13.4, 17.1 -> 13.8, 16.1 -> 16.2.  Classic CG, FP32
+    // and FP64: 43^3 18.8 -> 10.2 and 18.8 -> 15.0, 161^3 98 -> 47 and 125 -> 95, but
+    // 33^3 9.9 -> 10.2 and 10.6 -> 11.3; FP32 p(1) to p(3) where the resident solver
+    // does not run, 43^3 9.5 -> 7.9, 11.7 -> 9.2 and 14.0 -> 10.6.
     const int pitch = op == kOpStencil ? (int)align_up((size_t)A->st.nx, (size_t)want) : 0;
-    const bool pad = pad_lines && op == kOpStencil && vec == 1 && pitch != A->st.nx && A->st.nx >= 16 && !cg && l <= 3 &&
-                     !server && !resident && n > cluster_rows && (sc || (f32 && n >= (int64_t(1) << 18))) &&
+    const bool pad = pad_lines && op == kOpStencil && vec == 1 && pitch != A->st.nx && A->st.nx >= 16 && (cg || l <= 3) &&
+                     !resident && n > cluster_rows && (cg || f32 ? n >= kPadRows : sc) &&
                      (int64_t)pitch * A->st.ny * A->st.nz < (int64_t(1) << 31);
     const int64_t nv = pad ? (int64_t)pitch * A->st.ny * A->st.nz : n;   // rows of the solver's vectors
     if (pad) vec = want;
     // the sweep's operands copied a unit ahead
     const bool ahead = op == kOpStencil && !cg && l <= 2 && vec > 1 &&
                        (pad || (copies_ahead(f32, l, n) && !prm->dots_2l1));
-    const void *func = pad     ? kptr_st_pad(f32, l)
+    const void *func = pad     ? kptr_st_pad(f32, cg ? 0 : l)
                        : ahead ? kptr_st_ahead(f32, l)
                                : kernel_ptr(f32, op, vec, cg ? 0 : l, cg, sc, c32);
     if (!func) return fail(PLCG_ERR_UNIMPL, "no kernel for prec=%d op=%d vec=%d l=%d", prm->prec, op, vec, l);
@@ -1376,6 +1381,7 @@ struct ServerReq {
     double sigma[kMaxL] = {0};
     size_t bytes = 0;
     int64_t P = 0;
+    bool pad_lines = true;    // build_solve's
     double sm_share = 0.0;    // SMs its CTAs occupy: P / (resident CTAs per SM)
     int slot = -1;
     bool done = false;
@@ -1457,7 +1463,7 @@ static plcg_status server_launch(plcg_server *S, ServerReq &q)
     int per_sm = 0;
     size_t bytes = 0, o_out = 0;
     plcg_status s = build_solve<T>(q.A, q.b, q.x, &q.prm, q.sigma, (int)q.P, static_cast<char *>(ws),
-                                   &a, &func, &P, &per_sm, &bytes, &o_out, true);
+                                   &a, &func, &P, &per_sm, &bytes, &o_out, true, q.pad_lines);
     if (s == PLCG_OK) {
         CUDA_TRY(cudaEventRecord(S->ev0[q.slot], st));
         s = launch_built<T>(a, func, P, st);
@@ -1613,26 +1619,28 @@ extern "C" plcg_status plcg_submit(plcg_server *S, plcg_matrix *A, const double 
     int64_t P = 0;
     int per_sm = 0;
     size_t bytes = 0, o_out = 0;
-    if (prm->prec != PLCG_FP32_FP64DOT) {
-        SolveArgs<double> a;
-        st = build_solve<double>(A, b, x, &q->prm, q->sigma, 0, nullptr, &a, &func, &P, &per_sm, &bytes, &o_out, true);
-    } else {
+    auto build = [&](int ctas) -> plcg_status {
+        if (prm->prec != PLCG_FP32_FP64DOT) {
+            SolveArgs<double> a;
+            return build_solve<double>(A, b, x, &q->prm, q->sigma, ctas, nullptr, &a, &func, &P, &per_sm, &bytes, &o_out,
+                                       true, q->pad_lines);
+        }
         SolveArgs<float> a;
-        st = build_solve<float>(A, b, x, &q->prm, q->sigma, 0, nullptr, &a, &func, &P, &per_sm, &bytes, &o_out, true);
+        return build_solve<float>(A, b, x, &q->prm, q->sigma, ctas, nullptr, &a, &func, &P, &per_sm, &bytes, &o_out, true,
+                                  q->pad_lines);
+    };
+    for (bool pad_lines : {true, false}) {   // without padded lines where only they exceed the budget
+        q->pad_lines = pad_lines;
+        st = build(0);
+        if (st != PLCG_OK) return st;
+        const int cap = std::max(1, (per_sm * S->num_sms) / 2);
+        q->P = std::min<int64_t>(P, cap);
+        q->sm_share = (double)q->P / per_sm;
+        // recompute the byte count for the capped grid (partials scale with P)
+        st = build((int)q->P);
+        if (st != PLCG_OK) return st;
+        if (bytes <= S->budget) break;
     }
-    if (st != PLCG_OK) return st;
-    const int cap = std::max(1, (per_sm * S->num_sms) / 2);
-    q->P = std::min<int64_t>(P, cap);
-    q->sm_share = (double)q->P / per_sm;
-    // recompute the byte count for the capped grid (partials scale with P)
-    if (prm->prec != PLCG_FP32_FP64DOT) {
-        SolveArgs<double> a;
-        st = build_solve<double>(A, b, x, &q->prm, q->sigma, (int)q->P, nullptr, &a, &func, &P, &per_sm, &bytes, &o_out, true);
-    } else {
-        SolveArgs<float> a;
-        st = build_solve<float>(A, b, x, &q->prm, q->sigma, (int)q->P, nullptr, &a, &func, &P, &per_sm, &bytes, &o_out, true);
-    }
-    if (st != PLCG_OK) return st;
     q->bytes = bytes;
     std::lock_guard<std::mutex> lk(S->mu);
     if (S->stop) return fail(PLCG_ERR_INVALID, "server is shutting down");

@@ -2622,15 +2622,18 @@ finish:
 // vectors because the SpMV of step k reads neighbours of p_{k-1} while p_k is
 // written.  q = A p is in a.p; the recursive residual is r itself on the FP64
 // path and a.rc (FP32) on the FP32 path, whose inner iterate is the ring's
-// third vector.
+// third vector.  PAD: as in plcg_body; FP64 then keeps r and a correction of x as
+// FP32 does.
 // ------------------------------------------------------------------------
-template <typename T, int VEC, int OP, class Grp, int RPT = 1, typename CT = T>
+template <typename T, int VEC, int OP, class Grp, int RPT = 1, typename CT = T, bool PAD = false>
 __device__ void cg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
 {
     constexpr int UNIT = kBlock * VEC;
     constexpr int USWEEP = UNIT * RPT;
     constexpr bool kF32 = (sizeof(T) == 4);
-    const int64_t n = a.n;
+    constexpr bool kCorr = kF32 || PAD;   // the iterate is a segment's correction of x
+    static_assert(!PAD || (OP == kOpStencil && VEC > 1 && RPT == 1), "padded lines: stencils on the whole grid");
+    const int64_t n = PAD ? (int64_t)a.st.nx * a.st.ny * a.st.nz : a.n;   // rows of the solver's vectors
     const int64_t nunits = (n + UNIT - 1) / UNIT;
     const int tid = threadIdx.x;
     const T cC = (T)a.st.center, cO = (T)a.st.off;
@@ -2638,8 +2641,8 @@ __device__ void cg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
     T *q = a.p;
     std::conditional_t<(RPT > 1), StencilDesc, const StencilDesc &> st = a.st;
     const CsrDesc &csr = a.csr;
-    T *rc = kF32 ? a.rc : reinterpret_cast<T *>(a.r);
-    T *xi = kF32 ? a.zring + 2 * n : reinterpret_cast<T *>(a.x);
+    T *rc = kCorr ? a.rc : reinterpret_cast<T *>(a.r);
+    T *xi = kCorr ? a.zring + 2 * n : reinterpret_cast<T *>(a.x);
     const uint32_t nn = (uint32_t)n;   // n < 2^31
     // CSR on the whole grid, FP32: the SpMV sweep stages each unit's entries
     // (as in p(l)-CG).  FP64 CG runs without: its 3 CTAs per SM would not fit
@@ -2710,7 +2713,8 @@ __device__ void cg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
     } while (0)
 
     for (;;) {
-        residual_sweep<T, VEC, OP, Grp, CT>(a, a.st, s, grp);
+        if constexpr (PAD) residual_sweep<T, 1, OP, Grp, CT>(a, a.st0, s, grp);
+        else residual_sweep<T, VEC, OP, Grp, CT>(a, a.st, s, grp);
         grp.put_norms(a, s);
         spmvs++;
         CG_SYNC();
@@ -2719,9 +2723,9 @@ __device__ void cg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
         const double rn = sqrt(s.out[1]);
         last_rn = rn;
         if (normb == 0.0) {
-            for (int64_t u = grp.unit0(); u * kBlock < n; u += grp.ustep()) {
+            for (int64_t u = grp.unit0(); u * kBlock < a.n; u += grp.ustep()) {
                 const int64_t g = u * kBlock + tid;
-                if (g < n) a.x[g] = 0.0;
+                if (g < a.n) a.x[g] = 0.0;
             }
             status = kStOk;
             break;
@@ -2751,13 +2755,15 @@ __device__ void cg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
                 const int64_t g0 = u * UNIT + (int64_t)tid * VEC;
                 if (g0 >= n) continue;
                 T z[VEC], zero[VEC], zm[VEC];
+                const PadRows pr0 = pad_rows<PAD, VEC>(a, (uint32_t)g0);
 #pragma unroll
                 for (int v = 0; v < VEC; ++v) {
                     if constexpr (op_is_jacobi(OP)) {
                         z[v] = (T)(a.r[g0 + v] * __ldg(a.dinv64 + g0 + v));
                         zm[v] = z[v] * coef_cast<T>(__ldg(static_cast<const CT *>(csr.diag) + g0 + v));
                     } else {
-                        z[v] = (T)a.r[g0 + v];
+                        if constexpr (PAD) z[v] = v < pr0.cnt ? (T)a.r[pr0.user + v] : T(0);
+                        else z[v] = (T)a.r[g0 + v];
                         zm[v] = z[v];
                     }
                     zero[v] = T(0);
@@ -2773,6 +2779,20 @@ __device__ void cg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
             CG_SYNC();
             grp.template get_dots<1>(a, s, 0, s.raw);
             rr = s.raw[0];
+        } else if constexpr (PAD) {
+            for (int64_t u = grp.unit0(); u < nunits; u += grp.ustep()) {
+                const int64_t g0 = u * UNIT + (int64_t)tid * VEC;
+                if (g0 >= n) continue;
+                T z[VEC], zero[VEC];
+                const PadRows pr0 = pad_rows<PAD, VEC>(a, (uint32_t)g0);
+#pragma unroll
+                for (int v = 0; v < VEC; ++v) {
+                    z[v] = v < pr0.cnt ? (T)a.r[pr0.user + v] : T(0);
+                    zero[v] = T(0);
+                }
+                vst<T, VEC>(rc + g0, z);
+                vst<T, VEC>(xi + g0, zero);
+            }
         } else if constexpr (op_is_jacobi(OP)) {
             // FP64 path: z = M^{-1} r in r's place; rr = (r, M^{-1} r) = rn^2
             for (int64_t u = grp.unit0(); u < nunits; u += grp.ustep()) {
@@ -2858,6 +2878,11 @@ __device__ void cg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
                     if (g0 >= nn) continue;
                     T c[VEC], w[VEC];
                     op_apply<T, CT, VEC, OP>(st, csr, cC, cO, Ld1<T>{pn}, g0, c, w);
+                    if constexpr (PAD) {
+                        const int cnt = pad_rows<PAD, VEC>(a, g0).cnt;
+#pragma unroll
+                        for (int v = 0; v < VEC; ++v) w[v] = v < cnt ? w[v] : T(0);
+                    }
                     d1.add(c, w);
                     if constexpr (op_is_jacobi(OP)) w[0] *= __ldg(static_cast<const T *>(csr.dinv) + g0);
                     vst<T, VEC>(q + g0, w);
@@ -2960,6 +2985,11 @@ __device__ void cg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
                     for (int r = 0; r < RPT; ++r) {
                         if (g0[r] >= nn) continue;
                         vst<T, VEC>(pn + g0[r], c[r]);
+                        if constexpr (PAD) {
+                            const int cnt = pad_rows<PAD, VEC>(a, g0[r]).cnt;
+#pragma unroll
+                            for (int v = 0; v < VEC; ++v) w[r][v] = v < cnt ? w[r][v] : T(0);
+                        }
                         d1.add(c[r], w[r]);
                         if constexpr (op_is_jacobi(OP)) w[r][0] *= mi[r];   // q = M^{-1} A p
                         vst<T, VEC>(q + g0[r], w[r]);
@@ -3088,17 +3118,20 @@ __device__ void cg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
                 vst<T, VEC>(xi + g0, xv);
             }
         }
-        if (end == kSegNonfinite) { status = kStNonfinite; goto finish; }
-        if constexpr (kF32) {   // x += d
+        if (end == kSegNonfinite && kF32) { status = kStNonfinite; goto finish; }
+        if constexpr (kCorr) {   // x += d
             for (int64_t u = grp.unit0(); u < nunits; u += grp.ustep()) {
                 const int64_t g0 = u * UNIT + (int64_t)tid * VEC;
                 if (g0 >= n) continue;
                 T xv[VEC];
                 vld<T, VEC>(xi + g0, xv);
+                const PadRows pr0 = pad_rows<PAD, VEC>(a, (uint32_t)g0);
 #pragma unroll
-                for (int v = 0; v < VEC; ++v) a.x[g0 + v] += (double)xv[v];
+                for (int v = 0; v < VEC; ++v)
+                    if (!PAD || v < pr0.cnt) a.x[pr0.user + v] += (double)xv[v];
             }
         }
+        if (end == kSegNonfinite) { status = kStNonfinite; goto finish; }
         CG_SYNC();
     }
 finish:
@@ -3135,13 +3168,13 @@ plcg_kernel(SolveArgs<T> a)
     plcg_body<T, L, VEC, OP, GridGroup<T>, 1, SC, CT, false, PIPE, PAD>(a, s, grp);
 }
 
-template <typename T, int VEC, int OP, typename CT = T>
+template <typename T, int VEC, int OP, typename CT = T, bool PAD = false>
 __global__ void __launch_bounds__(kBlock, 3) cg_kernel(SolveArgs<T> a)
 {
     __shared__ Smem<T> s;
     GridGroup<T> grp;
     if (threadIdx.x == 0) s.quit = 0;
-    cg_body<T, VEC, OP, GridGroup<T>, 1, CT>(a, s, grp);
+    cg_body<T, VEC, OP, GridGroup<T>, 1, CT, PAD>(a, s, grp);
 }
 
 // Small systems: the grid is one thread-block cluster (ClusterGroup), launched

@@ -55,10 +55,10 @@ def test_few_blocks(P, size, prec, l, ctas):
 
 
 @pytest.mark.parametrize("size", [(17, 30941), (30, 97, 183), (31, 131, 137), (65, 97, 91), (1025, 513)], ids=str)
-@pytest.mark.parametrize("prec,l", [(p, l) for p in ("fp64", "fp32") for l in (1, 2, 3)])
+@pytest.mark.parametrize("prec,l", [(p, l) for p in ("fp64", "fp32") for l in (0, 1, 2, 3)])
 @pytest.mark.parametrize("ctas", [0, 5])
 def test_padded_lines(P, size, prec, l, ctas):
-    """Lines that are not whole vectors, held at a padded pitch; from a guess that is not zero."""
+    """Lines that are not whole vectors, held at a padded pitch; from a guess that is not zero (l = 0: classic CG)."""
     import torch
     op, nz = grid(*size), (size + (1,))[2]
     rng = np.random.default_rng(3)
@@ -66,6 +66,7 @@ def test_padded_lines(P, size, prec, l, ctas):
     b = torch.tensor(W.rhs(op, xs), device="cuda")
     x = torch.tensor(rng.standard_normal(W.op_size(op)), device="cuda")
     A = P.Matrix(op)
-    r = A.solve(b, x, l=l, interval=interval(nz), rtol=RTOL, prec=prec, grid_ctas=ctas)
+    kw = dict(l=l, interval=interval(nz)) if l else dict(method="cg")
+    r = A.solve(b, x, rtol=RTOL, prec=prec, grid_ctas=ctas, **kw)
     A.close()
     check(x, torch.tensor(xs, device="cuda"), nz, r)
