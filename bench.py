@@ -146,13 +146,14 @@ def profiled_record(name: str):
     return d
 
 
-def passes_per_iter(l: int, method: str) -> int:
+def passes_per_iter(l: int, method: str, paired: bool = False) -> int:
     """Streaming passes over length-n vectors per iteration (fused sweep,
-    l+1 dots): 3 per basis (read 2, write 1) + 4 for p and x + extra dot
-    operands z^(l)_j for l >= 4; classic CG: 10."""
+    l+1 dots): 3 per basis (read 2, write 1) + 4 for p and x (paired: 2, they
+    pass every second iteration in the stencil sweeps other than FP64 p(1)) +
+    extra dot operands z^(l)_j for l >= 4; classic CG: 10."""
     if method == "cg":
         return 10
-    return 3 * (l + 1) + 4 + max(0, l - 3)
+    return 3 * (l + 1) + (2 if paired else 4) + max(0, l - 3)
 
 
 def dp_flops_per_point(l: int) -> int:
@@ -354,7 +355,7 @@ def run_ours(args):
             r = A.solve(b, xl, l=l, interval=interval, rtol=RTOL)
             sweep[f"l{l}"] = {"iters": r.iters, "time_to_rtol_s": round(r.seconds, 5),
                               "iters_per_s": round(r.iters / r.seconds, 1),
-                              "hbm_gbs": round(r.iters * passes_per_iter(l, "plcg") * 8 * n
+                              "hbm_gbs": round(r.iters * passes_per_iter(l, "plcg", l >= 2) * 8 * n
                                                / r.seconds / 1e9, 1)}
         extra["plcg_l_sweep_fp64"] = sweep
         # FP32 vectors with FP64 dots / scalars / refinement
@@ -366,7 +367,7 @@ def run_ours(args):
             r = A.solve(b, xf, l=l, interval=interval, rtol=RTOL, prec="fp32")
             xf_np = xf.cpu().numpy()
             err = float(np.linalg.norm(b_np - W.rhs(op, xf_np)) / np.linalg.norm(b_np))
-            byt = r.iters * passes_per_iter(l, "plcg") * 4 * n
+            byt = r.iters * passes_per_iter(l, "plcg", True) * 4 * n
             rec32 = profiled_record("plcg_3d_fp32_l1.json") if l == 1 else None
             mp[f"l{l}"] = {"iters": r.iters, "refinements": r.refinements,
                            "traffic": None if rec32 is None else
@@ -595,7 +596,7 @@ def other_configs(plcg, W, dev, hbm_peak, orc):
         lat = np.array([r.latency for r in res]) * 1e3   # launch start -> each system's result
         ok = sum(r.status == 0 for r in res)
         ll = kw.get("l", 1)
-        vec_passes = 10 if "method" in kw else 3 * (ll + 1) + 4
+        vec_passes = 10 if "method" in kw else 3 * (ll + 1) + 2
         byt = sum(W.op_size(s_["op"]) * r.iters for s_, r in zip(systems, res)) * vec_passes * 4
         d[name] = {"status": st, "converged": ok, "batch_time_s": round(best, 5),
                    "schedule": {"gang_size": sched[0], "large_work_factor": sched[1],

@@ -1955,7 +1955,12 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
     constexpr bool kOolScalar = kF32 && kGrid;
     // the next step's vector pointers are set while the CTA waits at the barrier
     constexpr bool kEarly = kGrid && L == 1;
-    constexpr bool kFast = kGrid || std::is_same<Grp, ClusterGroup<T>>::value;
+    // stored FP64 matrices keep one warp's order of the sums and the plain
+    // reciprocals: p(l)-CG on irregular ones (random CSR) is sensitive to the last
+    // bits of the scalars (another order moves single entries of x by 1e-8)
+    constexpr bool kFreeOrder = kF32 || OP == kOpStencil;
+    constexpr bool kSumAll = kGrid && kFreeOrder;
+    constexpr bool kFast = (kGrid || std::is_same<Grp, ClusterGroup<T>>::value) && kFreeOrder;
     // FP64 p(1)-CG keeps its bases scaled (see scalar_step_body): two FP64
     // multiplies per row fewer in the FP64-bound sweep
     constexpr bool kScaled = SC && kScaledBases<T, L>;
@@ -2593,10 +2598,10 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
                 if (tid == kBlock - 1) step_vectors<T, L>(s.cfb[(i + 1) & 1], a, (int)(i + 1));
             PLCG_SYNC();
             if (!la) {   // MPI_Wait(req(i+1-l)) and the scalar step, serially (warp 0)
-                if constexpr (kGrid)
+                if constexpr (kSumAll)
                     if (i + 1 >= L) grp.template get_dots_all<2 * L + 1>(a, s, (int)((i + 1 - L) % (L + 1)), s.raw);
                 if (tid < 32) {
-                    if constexpr (!kGrid)
+                    if constexpr (!kSumAll)
                         if (i + 1 >= L)
                             grp.template get_dots_warp<2 * L + 1>(a, s, (int)((i + 1 - L) % (L + 1)), s.raw);
                     if (tid == 0)
