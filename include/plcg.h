@@ -345,9 +345,12 @@ const char *plcg_version(void);
 /* Bound on the polls of every device-side wait (grid barrier, server
  * mailbox); 0 restores the default (about 2 s at 64 ns per poll). */
 void plcg_debug_set_poll_limit(uint64_t polls);
-/* 1: every grid barrier of the next solves waits for one arrival more than
+/* Not 0: every grid barrier of the next solves waits for one arrival more than
  * there are thread blocks, so the first wait runs out and the solve returns
- * PLCG_ERR_TIMEOUT (exercises the bounded-wait path); 0: off. */
+ * PLCG_ERR_TIMEOUT (exercises the bounded-wait path).  In the register-resident
+ * solver on > 0 makes the waits for the other blocks' dots run out from exchange
+ * number `on` on (1: the first, in the true residual), on < 0 the waits for
+ * neighbours' values from iteration -on - 1 of the first segment on.  0: off. */
 void plcg_debug_force_barrier_timeout(int on);
 
 /* Launch shape and flags of the calling thread's last single-system solve

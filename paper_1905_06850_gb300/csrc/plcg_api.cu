@@ -55,7 +55,7 @@ extern "C" const char *plcg_last_error(void) { return g_last_error.c_str(); }
 void plcg::set_last_error(const std::string &msg) { g_last_error = msg; }
 extern "C" const char *plcg_version(void) { return "plcg 0.1 (sm_103a)"; }
 extern "C" void plcg_debug_set_poll_limit(uint64_t polls) { g_poll_limit = polls; }
-extern "C" void plcg_debug_force_barrier_timeout(int on) { g_force_timeout = on ? 1 : 0; }
+extern "C" void plcg_debug_force_barrier_timeout(int on) { g_force_timeout = on; }
 
 // Systems of at most this many rows run on the cluster-resident solver
 // (p(l >= 2)-CG and classic CG; p(1)-CG up to half of it), 0: never; set by
@@ -699,6 +699,8 @@ static plcg_status build_solve(const plcg_matrix *A, const double *b, double *x,
     a.fp32 = f32 ? 1 : 0;
     a.poll_limit = poll_limit();
     a.force_timeout = g_force_timeout;
+    a.res_force = a.force_timeout > 0 ? (unsigned)a.force_timeout : ~0u;
+    a.res_force_z = a.force_timeout < 0 ? 0u - (unsigned)a.force_timeout : ~0u;
     // l >= 2: compute each iteration's scalars during the previous sweep where
     // that latency is a visible share of an iteration (smaller systems)
     a.lookahead = (!cg && l >= 2 && n < (int64_t(1) << 22)) ? 1 : 0;

@@ -127,6 +127,7 @@ struct SolveArgs {
     int stage;                // CSR kernels: stage each unit's entries (rows long enough to pay)
     unsigned long long *pkt;  // register-resident solver: the exchange packets (zeroed per launch)
     int res_nsw;              // ... and its sweeping threads per CTA (0: not that solver)
+    unsigned res_force, res_force_z;   // ... test hook: the exchange and the z tag from which on waits run out
     double *trace;            // CG: alpha_k, beta_k of the first segment (spectrum estimates), or null
     int trace_cap;            // pairs trace can hold
 };

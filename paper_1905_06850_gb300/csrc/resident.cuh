@@ -79,7 +79,11 @@ struct ResSmem {
     double arg, rg, gm, invd;        // crit -> post
     double X[32];                    // l = 1: res_coef_x by lane
     ResCoef<T, L> cf[2];
-    int fail;                        // a bounded wait of this CTA ran out, or another CTA gave up
+    // a bounded wait of this CTA ran out, or another CTA gave up: by the parity of
+    // the iteration (2: exchange2), written before and read after that
+    // iteration's CTA barrier.  A warp that is an iteration ahead writes the other
+    // one, so all warps of the CTA leave after the same barrier.
+    int fail[3];
 };
 
 __device__ __forceinline__ bool finite_bits(double v)
@@ -144,7 +148,7 @@ struct ResExch {
     unsigned long long *pkt;
     int P, rank, nd;            // CTAs, this CTA, doubles per packet
     unsigned long long limit;   // a poll is an L2 round trip of several loads: an eighth of the grid barrier's
-    int force;
+    unsigned force;             // test hook: waits of exchanges from this number on run out
     int *abort_flag;
     __device__ __forceinline__ unsigned long long *at(unsigned e, int cta, int q) const
     {
@@ -165,7 +169,7 @@ struct ResExch {
     __device__ __forceinline__ bool wait(unsigned e, int q0, double (&v)[kResChunks][NA]) const
     {
         const int lane = threadIdx.x & 31;
-        const unsigned want = e + (force ? 1u : 0u);
+        const unsigned want = e + (e >= force ? 1u : 0u);   // (no tag of this slot: those differ by kResSlots)
         const unsigned long long *p[kResChunks];
 #pragma unroll
         for (int k = 0; k < kResChunks; ++k) p[k] = at(e, min(lane + 32 * k, P - 1), q0);
@@ -498,7 +502,7 @@ __device__ __forceinline__ int res_loop0(ResSmem<T, L> &s, const ResExch &ex, un
             if (i >= 1) {   // graw, arg, 1 / sqrt(arg)
                 const int m = i - 1;
                 double w[kResChunks][1];
-                if (!ex.wait<1>(e0 + (unsigned)(i - 1), 1, w) && lane == 0) s.fail = 1;
+                if (!ex.wait<1>(e0 + (unsigned)(i - 1), 1, w) && lane == 0) s.fail[i & 1] = 1;
                 res_sum<1>(w, ex.P, &s.raw[1]);
                 res_bar_sync(1, 64);
                 // rows c-2 (the symmetry of G: g_{c-1,c-1}) and c-1 of column c = m + 1
@@ -520,7 +524,7 @@ __device__ __forceinline__ int res_loop0(ResSmem<T, L> &s, const ResExch &ex, un
                 res_end<T, L>(s, ci, m, graw, arg, s.gm);
             }
             res_bar_all();
-            if (s.fail) return -1;
+            if (s.fail[i & 1]) return -1;
             if (ci.end >= 0) return i;
             res_bar_sync(3, 32 + nsw);
             res_publish<2>(ex, e0 + (unsigned)i, s.red[i & 1], nw);
@@ -534,11 +538,11 @@ __device__ __forceinline__ int res_loop0(ResSmem<T, L> &s, const ResExch &ex, un
                 res_sum<L + 1>(w, ex.P, s.raw);
                 res_crit<T, L>(s, i + 1, kc, kn, join);
             } else {
-                if (lane == 0) s.fail = 1;
+                if (lane == 0) s.fail[i & 1] = 1;
                 join();
             }
             res_bar_all();
-            if (s.fail) return -1;
+            if (s.fail[i & 1]) return -1;
         }
     }
 }
@@ -554,7 +558,7 @@ __device__ __forceinline__ int res_loop1(ResSmem<T, L> &s, const ResExch &ex, un
             if (i >= 1) {
                 const int m = i - 1;
                 double w[kResChunks][1];
-                if (!ex.wait<1>(e0 + (unsigned)(i - 1), 0, w) && lane == 0) s.fail = 1;
+                if (!ex.wait<1>(e0 + (unsigned)(i - 1), 0, w) && lane == 0) s.fail[i & 1] = 1;
                 res_sum<1>(w, ex.P, &s.raw[0]);
                 res_bar_arrive(1, 64);
                 const double gm = fma(s.D, s.raw[0], s.A) * s.igmm;
@@ -564,7 +568,7 @@ __device__ __forceinline__ int res_loop1(ResSmem<T, L> &s, const ResExch &ex, un
                 res_bar_arrive(2, 64);
             }
             res_bar_all();
-            if (s.fail) return -1;
+            if (s.fail[i & 1]) return -1;
         }
         if (s.cf[i & 1].end >= 0) return i;
         if (lane == 0) {
@@ -577,7 +581,7 @@ __device__ __forceinline__ int res_loop1(ResSmem<T, L> &s, const ResExch &ex, un
             res_bar_sync(3, 32 + nsw);
             res_publish<L + 1>(ex, e0 + (unsigned)i, s.red[i & 1], nw);
             res_bar_all();
-            if (s.fail) return -1;
+            if (s.fail[i & 1]) return -1;
         }
     }
 }
@@ -682,12 +686,13 @@ __device__ __forceinline__ int res_loop_rows(ResSmem<T, L> &s, const ResExch &ex
             if (cf.end >= 0) break;
         }
         T nb[R];
-        if (!res_neighbours<T, R>(ex, rows, zb + (size_t)(i & 1) * nn * W, zt + (unsigned)i, nx, nxy, three, c, nb) &&
+        const unsigned zi = zt + (unsigned)i, want = zi | (zi >= a.res_force_z ? 0x40000000u : 0u);   // (a tag of none)
+        if (!res_neighbours<T, R>(ex, rows, zb + (size_t)(i & 1) * nn * W, want, nx, nxy, three, c, nb) &&
             lane == 0)
-            s.fail = 1;
+            s.fail[i & 1] = 1;
         if constexpr (L == 1) {
             res_bar_all();
-            if (s.fail) return -1;
+            if (s.fail[i & 1]) return -1;
             if (cf.end >= 0) break;
         }
         DotAcc<T, 1> dac[L + 1];
@@ -765,7 +770,7 @@ __device__ __forceinline__ int res_loop_rows(ResSmem<T, L> &s, const ResExch &ex
         }
         if constexpr (L >= 2) {
             res_bar_all();
-            if (s.fail) return -1;
+            if (s.fail[i & 1]) return -1;
         }
     }
     // ---- final vector update of the segment
@@ -802,12 +807,12 @@ __device__ __forceinline__ int res_loop_idle(ResSmem<T, L> &s)
     for (int i = 0;; ++i) {
         if constexpr (L == 1) {
             res_bar_all();
-            if (s.fail) return -1;
+            if (s.fail[i & 1]) return -1;
             if (s.cf[i & 1].end >= 0) return i;
         } else {
             if (s.cf[i & 1].end >= 0) return i;
             res_bar_all();
-            if (s.fail) return -1;
+            if (s.fail[i & 1]) return -1;
         }
     }
 }
@@ -825,7 +830,7 @@ __global__ void __launch_bounds__(kResBlock, 1) resident_kernel(SolveArgs<T> a)
     __shared__ ResSmem<T, L> s;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int nsw = a.res_nsw, nw = nsw >> 5;
-    const ResExch ex{a.pkt, (int)gridDim.x, (int)blockIdx.x, res_dots(L), a.poll_limit / 8 + 1, a.force_timeout,
+    const ResExch ex{a.pkt, (int)gridDim.x, (int)blockIdx.x, res_dots(L), a.poll_limit / 8 + 1, a.res_force,
                      &a.out->abort};
     const uint32_t nn = (uint32_t)a.n, nx = (uint32_t)a.st.nx, nxy = nx * (uint32_t)a.st.ny;
     const bool three = a.st.dim == 3;
@@ -854,7 +859,7 @@ __global__ void __launch_bounds__(kResBlock, 1) resident_kernel(SolveArgs<T> a)
     unsigned e = 0;            // number of the last exchange of dots
     unsigned zt = 1;           // tag of z^(l)_0 of the segment
     if (tid < L) s.sig[tid] = a.sigma[tid];
-    if (tid == 0) s.fail = 0;
+    if (tid == 0) s.fail[0] = s.fail[1] = s.fail[2] = 0;
 
     long long iters = 0, spmvs = 0, restarts = 0, refinements = 0, segments = 0;
     int last_end = kSegConverged;
@@ -879,10 +884,10 @@ __global__ void __launch_bounds__(kResBlock, 1) resident_kernel(SolveArgs<T> a)
             const bool ok = ex.wait<2>(e, 0, w);
             __threadfence();
             if (ok) res_sum<2>(w, ex.P, s.norms);
-            else if (lane == 0) s.fail = 1;
+            else if (lane == 0) s.fail[2] = 1;
         }
         __syncthreads();
-        return !s.fail;
+        return !s.fail[2];
     };
 
     for (;;) {
