@@ -21,7 +21,17 @@
  *   - The library copies matrix data into device memory it owns; that memory
  *     and every workspace are released by plcg_destroy.
  *   - A solve runs on the stream given at matrix creation (NULL = the legacy
- *     default stream) and returns after the stream has finished it.
+ *     default stream) and returns after the stream has finished it.  Solves of
+ *     matrices on streams of their own, from several host threads, run side by
+ *     side as far as their thread blocks fit the GPU.  p(l)-CG with l <= 3 on
+ *     stencils spreads over up to every SM (see plcg_set_cluster_rows): four
+ *     callers of up to 10^4 rows still run together (2D 100 x 100 p(2)-CG: 1660
+ *     solves of 200 iterations a second alone, 4940 from four), two up to about
+ *     3 x 10^4 rows, one above.  Where that is fewer than the whole-grid kernels
+ *     allow (FP32, 3 x 10^4 to 10^5 rows, three callers or more: 3D 40^3 p(1)-CG
+ *     1110 a second against 2100 on the grid, and 590 for one caller there), set
+ *     plcg_params.grid_ctas (1 << 20: the grid kernels at their full size), or
+ *     submit them to a server.
  *   - Every device-side wait in the library is bounded; when a bound expires
  *     the solve returns PLCG_ERR_TIMEOUT and the CUDA context stays usable.
  */

@@ -762,7 +762,7 @@ static plcg_status launch_built(const SolveArgs<T> &a0, const void *func, int64_
         cfg.numAttrs = 1;
         CUDA_TRY(cudaLaunchKernelExC(&cfg, func, args));
     } else {
-        CUDA_TRY(cudaLaunchCooperativeKernel(func, dim3((unsigned)P), dim3(a.res_nsw ? kResBlock : kBlock), args, a.dsmem, stream));
+        CUDA_TRY(cudaLaunchCooperativeKernel(func, dim3((unsigned)P), dim3((unsigned)(a.res_nsw ? 64 + a.res_nsw : kBlock)), args, a.dsmem, stream));
     }
     return PLCG_OK;
 }

@@ -800,26 +800,9 @@ __device__ __forceinline__ int res_loop_rows(ResSmem<T, L> &s, const ResExch &ex
     return i;
 }
 
-// A warp without rows.
-template <typename T, int L>
-__device__ __forceinline__ int res_loop_idle(ResSmem<T, L> &s)
-{
-    for (int i = 0;; ++i) {
-        if constexpr (L == 1) {
-            res_bar_all();
-            if (s.fail[i & 1]) return -1;
-            if (s.cf[i & 1].end >= 0) return i;
-        } else {
-            if (s.cf[i & 1].end >= 0) return i;
-            res_bar_all();
-            if (s.fail[i & 1]) return -1;
-        }
-    }
-}
-
 // ------------------------------------------------------------------------
 // A whole solve.  Threads 0 .. 31: warp 0; 32 .. 63: warp 1; 64 .. 64 + nsw -
-// 1: R rows each.  Cooperative launch, at most 32 kResChunks CTAs.
+// 1, the last: R rows each.  Cooperative launch, at most 32 kResChunks CTAs.
 // ------------------------------------------------------------------------
 template <typename T, int L, int R>
 __global__ void __launch_bounds__(kResBlock, 1) resident_kernel(SolveArgs<T> a)
@@ -835,7 +818,7 @@ __global__ void __launch_bounds__(kResBlock, 1) resident_kernel(SolveArgs<T> a)
     const uint32_t nn = (uint32_t)a.n, nx = (uint32_t)a.st.nx, nxy = nx * (uint32_t)a.st.ny;
     const bool three = a.st.dim == 3;
     const T kc = (T)a.st.center, kn = (T)a.st.off;
-    const bool sweeps = tid >= 64 && tid < 64 + nsw;
+    const bool sweeps = tid >= 64;
     ResRows<R> rows;
 #pragma unroll
     for (int r = 0; r < R; ++r) {
@@ -942,8 +925,7 @@ __global__ void __launch_bounds__(kResBlock, 1) resident_kernel(SolveArgs<T> a)
         int i;
         if (warp == 0) i = res_loop0<T, L>(s, ex, e0, nsw, kc, kn);
         else if (warp == 1) i = res_loop1<T, L>(s, ex, e0, nsw, kc, kn, rn, tau, budget);
-        else if (sweeps) i = res_loop_rows<T, L, R>(s, ex, a, rows, zt, nsw, rn, kc, kn);
-        else i = res_loop_idle<T, L>(s);
+        else i = res_loop_rows<T, L, R>(s, ex, a, rows, zt, nsw, rn, kc, kn);
         if (i < 0) { status = kStTimeout; break; }
         e = e0 + (unsigned)i;
         zt += (unsigned)i + 2u;
