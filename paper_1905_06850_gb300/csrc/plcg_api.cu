@@ -7,6 +7,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -82,7 +83,7 @@ static bool copies_ahead(bool f32, int l, int64_t n)
     if (!f32) return n >= (5 << 18);
     return l != 1 || n < (7 << 18) || n >= (3 << 20);
 }
-static int64_t g_cluster_rows = kClusterRowsDefault;
+static std::atomic<int64_t> g_cluster_rows{kClusterRowsDefault};
 
 extern "C" plcg_status plcg_set_cluster_rows(int64_t max_rows)
 {
@@ -483,14 +484,24 @@ static plcg_status ensure_ws(plcg_matrix *A, size_t bytes)
 
 // Layout of one solve's workspace and its kernel arguments.  With base ==
 // nullptr only the sizes are computed; *bytes is the workspace size and
-// *out_off the offset of the result record inside it.  pad_lines = false: no
-// padded lines (they take up to a fifth more workspace).
+// *out_off the offset of the result record inside it.
+//
+// What a solve's layout depends on besides its arguments: taken once per solve,
+// so that the workspace that is sized and the one that is used later (a served
+// request's by another thread) are laid out the same whatever
+// plcg_set_cluster_rows has been given in between.
+struct BuildOpts {
+    int64_t cluster_rows = g_cluster_rows.load();
+    bool server = false;
+    bool pad_lines = true;   // false: no padded lines (they take up to a fifth more workspace)
+};
+
 template <typename T>
 static plcg_status build_solve(const plcg_matrix *A, const double *b, double *x,
                                const plcg_params *prm, const double *sigma, int max_ctas,
                                char *base, SolveArgs<T> *args, const void **func_out,
                                int64_t *P_out, int *per_sm_out, size_t *bytes, size_t *out_off,
-                               bool server = false, bool pad_lines = true)
+                               const BuildOpts &opt)
 {
     const int64_t n = A->n;
     const int l = prm->l;
@@ -506,9 +517,9 @@ static plcg_status build_solve(const plcg_matrix *A, const double *b, double *x,
     // state in registers (resident.cuh), 32 rows per CTA at least, up to 4 per
     // thread; a cluster limit raised above its default asks for the cluster
     // path instead, and a server keeps the smaller footprint of the others
-    const int64_t cluster_rows = cg || l >= 2 ? g_cluster_rows : g_cluster_rows / 2;
+    const int64_t cluster_rows = cg || l >= 2 ? opt.cluster_rows : opt.cluster_rows / 2;
     const bool resident = op == kOpStencil && !cg && l <= 3 && !prm->dots_2l1 && prm->grid_ctas == 0 && max_ctas == 0 &&
-                          !server && !(g_cluster_rows > kClusterRowsDefault && n <= cluster_rows) &&
+                          !opt.server && !(opt.cluster_rows > kClusterRowsDefault && n <= cluster_rows) &&
                           n <= (int64_t)std::min(A->num_sms, 32 * kResChunks) * kResSweep * 4;
     // Stencil rows per thread: 16 bytes of a vector (rows in one x-line),
     // except FP64 systems of at most kVec1Rows rows, which take one row per
@@ -536,7 +547,7 @@ static plcg_status build_solve(const plcg_matrix *A, const double *b, double *x,
     // 33^3 9.9 -> 10.2 and 10.6 -> 11.3; FP32 p(1) to p(3) where the resident solver
     // does not run, 43^3 9.5 -> 7.9, 11.7 -> 9.2 and 14.0 -> 10.6.
     const int pitch = op == kOpStencil ? (int)align_up((size_t)A->st.nx, (size_t)want) : 0;
-    const bool pad = pad_lines && op == kOpStencil && vec == 1 && pitch != A->st.nx && A->st.nx >= 16 && (cg || l <= 3) &&
+    const bool pad = opt.pad_lines && op == kOpStencil && vec == 1 && pitch != A->st.nx && A->st.nx >= 16 && (cg || l <= 3) &&
                      !resident && n > cluster_rows && (cg || f32 ? n >= kPadRows : sc) &&
                      (int64_t)pitch * A->st.ny * A->st.nz < (int64_t(1) << 31);
     const int64_t nv = pad ? (int64_t)pitch * A->st.ny * A->st.nz : n;   // rows of the solver's vectors
@@ -791,17 +802,18 @@ static plcg_status run_solve(plcg_matrix *A, const double *b, double *x, const p
     int64_t P = 0;
     int per_sm = 0;
     size_t bytes = 0, o_out = 0;
-    plcg_status st = build_solve<T>(A, b, x, prm, sigma, 0, nullptr, &a, &func, &P, &per_sm, &bytes, &o_out);
+    BuildOpts opt;
+    plcg_status st = build_solve<T>(A, b, x, prm, sigma, 0, nullptr, &a, &func, &P, &per_sm, &bytes, &o_out, opt);
     if (st != PLCG_OK) return st;
     st = ensure_ws(A, bytes);
-    const bool pad_lines = st != PLCG_ERR_NOMEM;
-    if (!pad_lines) {   // without padded lines, if that needs less
-        st = build_solve<T>(A, b, x, prm, sigma, 0, nullptr, &a, &func, &P, &per_sm, &bytes, &o_out, false, false);
+    opt.pad_lines = st != PLCG_ERR_NOMEM;
+    if (!opt.pad_lines) {   // without padded lines, if that needs less
+        st = build_solve<T>(A, b, x, prm, sigma, 0, nullptr, &a, &func, &P, &per_sm, &bytes, &o_out, opt);
         if (st == PLCG_OK) st = ensure_ws(A, bytes);
     }
     if (st != PLCG_OK) return st;
     st = build_solve<T>(A, b, x, prm, sigma, 0, static_cast<char *>(A->ws.mem), &a, &func, &P,
-                        &per_sm, &bytes, &o_out, false, pad_lines);
+                        &per_sm, &bytes, &o_out, opt);
     if (st != PLCG_OK) return st;
     a.trace = trace;
     a.trace_cap = trace_cap;
@@ -901,16 +913,17 @@ static plcg_status run_solve_fixed(const plcg_matrix *A, const double *b, double
     int64_t P = 0;
     int per_sm = 0;
     size_t bytes = 0, o_out = 0;
-    plcg_status st = build_solve<T>(A, b, x, prm, sigma, 0, nullptr, &a, &func, &P, &per_sm, &bytes, &o_out);
-    const bool pad_lines = st != PLCG_OK || bytes <= cap;
-    if (!pad_lines)
-        st = build_solve<T>(A, b, x, prm, sigma, 0, nullptr, &a, &func, &P, &per_sm, &bytes, &o_out, false, false);
+    BuildOpts opt;
+    plcg_status st = build_solve<T>(A, b, x, prm, sigma, 0, nullptr, &a, &func, &P, &per_sm, &bytes, &o_out, opt);
+    opt.pad_lines = st != PLCG_OK || bytes <= cap;
+    if (!opt.pad_lines)
+        st = build_solve<T>(A, b, x, prm, sigma, 0, nullptr, &a, &func, &P, &per_sm, &bytes, &o_out, opt);
     if (st != PLCG_OK) return st;
     if (bytes > cap)
         return fail(PLCG_ERR_INVALID,
                     "%s: this solve needs %zu bytes of scratch; the fixed no-allocation scratch holds %zu bytes "
                     "(use plcg_solve)", who, bytes, cap);
-    st = build_solve<T>(A, b, x, prm, sigma, 0, base, &a, &func, &P, &per_sm, &bytes, &o_out, false, pad_lines);
+    st = build_solve<T>(A, b, x, prm, sigma, 0, base, &a, &func, &P, &per_sm, &bytes, &o_out, opt);
     if (st != PLCG_OK) return st;
     st = launch_built<T>(a, func, P, A->stream);
     if (st != PLCG_OK) return st;
@@ -1383,7 +1396,7 @@ struct ServerReq {
     double sigma[kMaxL] = {0};
     size_t bytes = 0;
     int64_t P = 0;
-    bool pad_lines = true;    // build_solve's
+    BuildOpts opt;            // build_solve's, as at submission
     double sm_share = 0.0;    // SMs its CTAs occupy: P / (resident CTAs per SM)
     int slot = -1;
     bool done = false;
@@ -1465,7 +1478,7 @@ static plcg_status server_launch(plcg_server *S, ServerReq &q)
     int per_sm = 0;
     size_t bytes = 0, o_out = 0;
     plcg_status s = build_solve<T>(q.A, q.b, q.x, &q.prm, q.sigma, (int)q.P, static_cast<char *>(ws),
-                                   &a, &func, &P, &per_sm, &bytes, &o_out, true, q.pad_lines);
+                                   &a, &func, &P, &per_sm, &bytes, &o_out, q.opt);
     if (s == PLCG_OK) {
         CUDA_TRY(cudaEventRecord(S->ev0[q.slot], st));
         s = launch_built<T>(a, func, P, st);
@@ -1621,18 +1634,19 @@ extern "C" plcg_status plcg_submit(plcg_server *S, plcg_matrix *A, const double 
     int64_t P = 0;
     int per_sm = 0;
     size_t bytes = 0, o_out = 0;
+    q->opt.server = true;
     auto build = [&](int ctas) -> plcg_status {
         if (prm->prec != PLCG_FP32_FP64DOT) {
             SolveArgs<double> a;
             return build_solve<double>(A, b, x, &q->prm, q->sigma, ctas, nullptr, &a, &func, &P, &per_sm, &bytes, &o_out,
-                                       true, q->pad_lines);
+                                       q->opt);
         }
         SolveArgs<float> a;
-        return build_solve<float>(A, b, x, &q->prm, q->sigma, ctas, nullptr, &a, &func, &P, &per_sm, &bytes, &o_out, true,
-                                  q->pad_lines);
+        return build_solve<float>(A, b, x, &q->prm, q->sigma, ctas, nullptr, &a, &func, &P, &per_sm, &bytes, &o_out,
+                                  q->opt);
     };
     for (bool pad_lines : {true, false}) {   // without padded lines where only they exceed the budget
-        q->pad_lines = pad_lines;
+        q->opt.pad_lines = pad_lines;
         st = build(0);
         if (st != PLCG_OK) return st;
         const int cap = std::max(1, (per_sm * S->num_sms) / 2);
