@@ -363,6 +363,10 @@ void plcg_debug_set_poll_limit(uint64_t polls);
  * neighbours' values from iteration -on - 1 of the first segment on.  0: off. */
 void plcg_debug_force_barrier_timeout(int on);
 
+/* Workspaces of single solves and of served requests above `bytes` are refused
+ * as the device refuses memory that it does not have; 0: off. */
+void plcg_debug_limit_workspace(uint64_t bytes);
+
 /* Launch shape and flags of the calling thread's last single-system solve
  * launch (plcg_solve, plcg_solve_host, plcg_estimate_interval,
  * plcg_solve_stencil_noalloc), so that tests can check that two entry

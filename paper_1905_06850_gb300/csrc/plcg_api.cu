@@ -165,6 +165,7 @@ struct plcg_matrix {
     int device = 0;
     int num_sms = 0;
     Workspace ws;
+    size_t pad_refused = 0;       // bytes of a workspace with padded lines that the device did not have (0: none)
     double *b_dev = nullptr, *x_dev = nullptr;   // plcg_solve_host staging
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     DevResult *host_res = nullptr;              // pinned
@@ -467,6 +468,23 @@ static void resolve_shifts(const plcg_matrix *A, const plcg_params *prm, double 
         for (int k = 0; k < prm->l; ++k) sigma[k] *= A->st.center;
 }
 
+// Test hook: solver workspaces above this many bytes are refused as the device
+// refuses what it does not have (0: off).
+static std::atomic<uint64_t> g_ws_limit{0};
+extern "C" void plcg_debug_limit_workspace(uint64_t bytes) { g_ws_limit = bytes; }
+
+// cudaMalloc of a workspace, or on a stream.  A refusal leaves no pending error
+// of the runtime's: solves try again with less, and the next kernel launch would
+// report it.
+static cudaError_t ws_alloc(void **mem, size_t bytes, const cudaStream_t *stream = nullptr)
+{
+    const uint64_t limit = g_ws_limit.load();
+    const size_t ask = limit && bytes > limit ? SIZE_MAX / 4 : bytes;
+    const cudaError_t e = stream ? cudaMallocAsync(mem, ask, *stream) : cudaMalloc(mem, ask);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
+}
+
 static plcg_status ensure_ws(plcg_matrix *A, size_t bytes)
 {
     if (A->ws.bytes >= bytes) return PLCG_OK;
@@ -476,7 +494,7 @@ static plcg_status ensure_ws(plcg_matrix *A, size_t bytes)
         A->ws.mem = nullptr;
         A->ws.bytes = 0;
     }
-    CUDA_TRY(cudaMalloc(&A->ws.mem, bytes));
+    CUDA_TRY(ws_alloc(&A->ws.mem, bytes));
     A->ws.bytes = bytes;
     return PLCG_OK;
 }
@@ -805,11 +823,18 @@ static plcg_status run_solve(plcg_matrix *A, const double *b, double *x, const p
     BuildOpts opt;
     plcg_status st = build_solve<T>(A, b, x, prm, sigma, 0, nullptr, &a, &func, &P, &per_sm, &bytes, &o_out, opt);
     if (st != PLCG_OK) return st;
-    st = ensure_ws(A, bytes);
-    opt.pad_lines = st != PLCG_ERR_NOMEM;
-    if (!opt.pad_lines) {   // without padded lines, if that needs less
-        st = build_solve<T>(A, b, x, prm, sigma, 0, nullptr, &a, &func, &P, &per_sm, &bytes, &o_out, opt);
-        if (st == PLCG_OK) st = ensure_ws(A, bytes);
+    // Without padded lines, if that needs less, where the device does not hold the
+    // padded workspace; what it has refused this handle once is not asked for again
+    // (the smaller workspace would be given back for it each time).
+    const size_t padded = bytes;
+    const bool known = A->pad_refused && padded >= A->pad_refused && padded > A->ws.bytes;
+    st = known ? PLCG_ERR_NOMEM : ensure_ws(A, padded);
+    if (st == PLCG_ERR_NOMEM) {
+        opt.pad_lines = false;
+        const plcg_status st2 = build_solve<T>(A, b, x, prm, sigma, 0, nullptr, &a, &func, &P, &per_sm, &bytes, &o_out, opt);
+        if (st2 != PLCG_OK) return st2;
+        if (known || bytes < padded) st = ensure_ws(A, bytes);
+        if (st == PLCG_OK && bytes < padded) A->pad_refused = known ? std::min(A->pad_refused, padded) : padded;
     }
     if (st != PLCG_OK) return st;
     st = build_solve<T>(A, b, x, prm, sigma, 0, static_cast<char *>(A->ws.mem), &a, &func, &P,
@@ -1471,7 +1496,20 @@ static plcg_status server_launch(plcg_server *S, ServerReq &q)
 {
     const cudaStream_t st = S->streams[q.slot];
     void *ws = nullptr;
-    CUDA_TRY(cudaMallocAsync(&ws, q.bytes, st));
+    cudaError_t e = ws_alloc(&ws, q.bytes, &st);
+    if (e == cudaErrorMemoryAllocation && q.opt.pad_lines) {   // without padded lines, if that needs less
+        q.opt.pad_lines = false;
+        SolveArgs<T> a;
+        const void *func = nullptr;
+        int64_t P = 0;
+        int per_sm = 0;
+        size_t less = 0, o_out = 0;
+        const plcg_status s = build_solve<T>(q.A, q.b, q.x, &q.prm, q.sigma, (int)q.P, nullptr, &a, &func, &P, &per_sm,
+                                             &less, &o_out, q.opt);
+        if (s != PLCG_OK) return s;
+        if (less < q.bytes) e = ws_alloc(&ws, less, &st);
+    }
+    CUDA_TRY(e);
     SolveArgs<T> a;
     const void *func = nullptr;
     int64_t P = 0;

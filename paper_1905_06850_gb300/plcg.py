@@ -100,6 +100,7 @@ SIGNATURES = {
     "plcg_version": (C.c_char_p, []),
     "plcg_debug_set_poll_limit": (None, [C.c_uint64]),
     "plcg_debug_force_barrier_timeout": (None, [C.c_int]),
+    "plcg_debug_limit_workspace": (None, [C.c_uint64]),
     "plcg_debug_last_launch": (None, [C.POINTER(plcg_launch_info)]),
     "plcg_debug_server_admission": (C.c_int, [C.c_int, _VP, _VP, _VP, C.c_uint64, C.c_double, C.c_int,
                                               C.c_int, _VP]),
