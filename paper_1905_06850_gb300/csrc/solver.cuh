@@ -274,7 +274,7 @@ __device__ __forceinline__ void warp_columns_sum(const double *part, int count, 
 #pragma unroll
     for (int q = 0; q < NA; ++q) v[q] = 0.0;
     int c = lane;
-    for (; c + 96 < count; c += 128) {
+    for (; c - lane + 128 <= count; c += 128) {   // (the same trips for all lanes: a part batch would run beside the loop below)
         double w[4][NA];
 #pragma unroll
         for (int j = 0; j < 4; ++j)
@@ -1164,7 +1164,7 @@ struct SweepCoef {
 };
 
 template <typename T>
-struct Smem {
+struct alignas(16) Smem {   // (what follows it in the batched kernel stays 16-byte aligned: 8 bytes more, FP32 p(1)-CG 266 -> 285 us)
     double red[(kBlock / 32) * kMaxDots];
     double out[kMaxDots + 2];
     double raw[kMaxDots];
@@ -1181,8 +1181,6 @@ struct Smem {
     double raw2[kMaxDots];           // the scalar warp's copy of a reduced dot column
     Coef<T> cfb[2];                  // coefficients of iterations i (i & 1) and i + 1
     T zxr[2], ppr[2];                // K6 in pairs: zx and pp of step m in slot (m >> 1) & 1, m odd
-    long long stg_e0;                // CSR staging: global position of the unit's first staged entry
-    int stg_on;                      // CSR staging: this unit's entries are in shared memory
     int ok;
     int quit;                        // whole grid: a bulk copy of this CTA did not land in time
 };
@@ -1959,12 +1957,25 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
     // reciprocals: p(l)-CG on irregular ones (random CSR) is sensitive to the last
     // bits of the scalars (another order moves single entries of x by 1e-8)
     constexpr bool kFreeOrder = kF32 || OP == kOpStencil;
-    constexpr bool kSumAll = kGrid && kFreeOrder;
-    constexpr bool kFast = (kGrid || std::is_same<Grp, ClusterGroup<T>>::value) && kFreeOrder;
+    // stencils of l > 4: one warp's sums as well (the CTA's take 2 (l + 1) registers
+    // more of the 128: FP64 p(8)-CG spilled 444 bytes instead of 224, FP32 131^3
+    // p(5)-CG 91.4 us per iteration instead of 86.6)
+    constexpr bool kSumAll = kGrid && kFreeOrder && (L <= 4 || OP != kOpStencil);
+    // where the scalar step is out of line or spills (l > 4), the call in the fast
+    // reciprocals' fallback costs the sweep its registers (FP32 CSR 96^3 p(2)-CG 80.0
+    // us per iteration without, 91.0 with; FP64 2D 32^2 p(8)-CG 15.3 and 15.8)
+    constexpr bool kFast =
+        (kGrid || std::is_same<Grp, ClusterGroup<T>>::value) && kFreeOrder && !kOolScalar && L <= 4;
     // FP64 p(1)-CG keeps its bases scaled (see scalar_step_body): two FP64
     // multiplies per row fewer in the FP64-bound sweep
     constexpr bool kScaled = SC && kScaledBases<T, L>;
     constexpr bool kPair = kPairK6<T, L, VEC, OP, Grp>;
+    // the final update loads p where it uses it, else ahead of its branches: there it
+    // costs the 27-point sweeps of l = 1 and, with FP64 values, l = 2 registers (FP64
+    // 96^3 p(1)-CG 93.4 us per iteration, 87.9 without; p(2) 154.4, 147.6); those of
+    // FP32 values and of l > 2 gain by it as often as they lose
+    constexpr bool kLateP = !kPair && (L == 1 || (L == 2 && sizeof(CT) == 8));
+    constexpr int kMoves = kPair ? 2 : 4;   // the k6 with which p and x pass through memory
     // CSR on the whole grid: each sweep unit's entries are bulk-copied into
     // shared memory (one contiguous range per unit) before its rows are read
     constexpr bool kStage = op_is_csr(OP) && std::is_same<Grp, GridGroup<T>>::value && RPT == 1;
@@ -2139,7 +2150,8 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
                         if (g0 >= n) continue;
                         T xv[VEC], pv[VEC];
                         vld<T, VEC>(xi + g0, xv);
-                        if (pend || cf.f1 != T(0) || cf.fmode == 1) vld<T, VEC>(a.p + g0, pv);
+                        if constexpr (!kLateP)
+                            if (pend || cf.f1 != T(0) || cf.fmode == 1) vld<T, VEC>(a.p + g0, pv);
                         if (pend) {
                             T wv[VEC];
                             vld<T, VEC>(cf.prv[0] + g0, wv);
@@ -2151,6 +2163,7 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
                         }
                         if (cf.fmode == 0) {
                             if (cf.f1 != T(0)) {
+                                if constexpr (kLateP) vld<T, VEC>(a.p + g0, pv);
 #pragma unroll
                                 for (int v = 0; v < VEC; ++v) xv[v] = fma(cf.f1, pv[v], xv[v]);
                             }
@@ -2158,6 +2171,7 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
                             T vv[VEC];
                             vld<T, VEC>(cf.v0 + g0, vv);
                             if (cf.fmode == 1) {
+                                if constexpr (kLateP) vld<T, VEC>(a.p + g0, pv);
 #pragma unroll
                                 for (int v = 0; v < VEC; ++v) {
                                     xv[v] = fma(cf.f1, pv[v], xv[v]);
@@ -2251,6 +2265,11 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
                 constexpr int K6 = decltype(k6_tag)::value;   // 2, 3 or 4, 0: read from C
                 const bool rec = S || C.mode == 1;
                 const int k6 = K6 ? K6 : C.k6;
+                // does this sweep move p and x (and p only: k6 = 1)?  (In one cluster or
+                // one CTA a single comparison: 2D 100^2 p(2)-CG, 2l+1 dots, 7.52 -> 7.43 us
+                // per iteration; on the grid that costs FP32 131^3 p(5)-CG 88 -> 93.)
+                auto moves = [&] { return kGrid ? (k6 == 2 || k6 == 4) : k6 == kMoves; };
+                auto moves_p = [&] { return kGrid ? (k6 != 0 && k6 != 3) : (k6 == 1 || k6 == kMoves); };
                 const bool prev0 = S || C.prev0;
                 int since_flush = 0;
                 // 27-point tiles: the first unit's copies start here, each
@@ -2435,7 +2454,7 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
                                 }
                             }
                         }
-                        if (k6 == 2 || k6 == 4) {
+                        if (moves()) {
                             vld<T, VEC>(pvec + g0[r], pv[r]);
                             vld<T, VEC>(xi + g0[r], xv[r]);
                         }
@@ -2502,7 +2521,7 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
                         if (k6 == 1) {
 #pragma unroll
                             for (int v = 0; v < VEC; ++v) pv[r][v] = cur[r][0][v];
-                        } else if (k6 != 0 && k6 != 3) {
+                        } else if (moves_p()) {
                             if (kPair)
 #pragma unroll
                                 for (int v = 0; v < VEC; ++v) {
@@ -2523,8 +2542,8 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
 #pragma unroll
                             for (int k = 0; k < L; ++k) vst<T, VEC>(C.nw[k] + g0[r], nw[k]);
                         }
-                        if (k6 != 0 && k6 != 3) vst<T, VEC>(pvec + g0[r], pv[r]);
-                        if (k6 == 2 || k6 == 4) vst<T, VEC>(xi + g0[r], xv[r]);
+                        if (moves_p()) vst<T, VEC>(pvec + g0[r], pv[r]);
+                        if (moves()) vst<T, VEC>(xi + g0[r], xv[r]);
                         // -- K5: partial dot products with u_{i+1} = M z^(l)_{i+1}
                         // (M = I: z^(l)_{i+1} itself)
                         T uM[VEC];
