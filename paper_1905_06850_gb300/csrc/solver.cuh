@@ -2017,6 +2017,7 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
                             (op_is_var27(OP) ? kF32 && L <= 2
                                              : OP == kOpStencil && (PIPE || (!kF32 && VEC > 1 && L <= 4) || L == 3 || L == 4));
     constexpr bool kPipe = PIPE;
+    static_assert(!(kTile && kPair), "27-point tiles hold p and x of every sweep");
     static_assert(!PIPE || (OP == kOpStencil && VEC > 1 && kGrid && RPT == 1), "copies ahead: 16-byte rows");
     static_assert(!PAD || (OP == kOpStencil && VEC > 1 && kGrid), "padded lines: stencils on the whole grid");
     constexpr bool kCorr = kF32 || PAD;   // the iterate is a segment's correction of x
@@ -2283,8 +2284,8 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
                     if (j == 0) return C.zl_prev;
                     if (j <= L) return C.cur[j - 1];
                     if (j <= 2 * L) return C.prv[j - 1 - L];
-                    if (j == 2 * L + 1) return k6 != 3 ? pvec : nullptr;
-                    if (j == 2 * L + 2) return k6 != 3 ? static_cast<const T *>(xi) : nullptr;
+                    if (j == 2 * L + 1) return pvec;
+                    if (j == 2 * L + 2) return static_cast<const T *>(xi);
                     return static_cast<const T *>(csr.dinv);
                 };
                 // stage unit uu (if it exists) in buffer bb
@@ -2416,10 +2417,8 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
                                     cur[r][k][0] = tile.vec(tb, 1 + k)[t];
                                     pk[r][k][0] = tile.vec(tb, 1 + L + k)[t];
                                 }
-                                if (k6 != 3) {
-                                    pv[r][0] = tile.vec(tb, 2 * L + 1)[t];
-                                    xv[r][0] = tile.vec(tb, 2 * L + 2)[t];
-                                }
+                                pv[r][0] = tile.vec(tb, 2 * L + 1)[t];
+                                xv[r][0] = tile.vec(tb, 2 * L + 2)[t];
                                 if constexpr (op_is_jacobi(OP)) {
                                     c[r][0] = tile.vec(tb, 2 * L + 3)[t];   // 1 / a_gg for now
                                     dg[r] = tile.diag(tb, t);                // a_gg: the diagonal slot
@@ -2584,7 +2583,7 @@ __device__ void plcg_body(const SolveArgs<T> &a, Smem<T> &s, Grp &grp)
             // (one loop for both where a sweep is short: its instructions are
             // fetched anew in every launch, and a second loop's cost more than
             // the test)
-            constexpr bool kSplit = std::is_same<Grp, BlockGroup<T>>::value || VEC > 1 || kTile;
+            constexpr bool kSplit = std::is_same<Grp, BlockGroup<T>>::value || VEC > 1;
             if (steady) {
                 if constexpr (!kPair) sweep(std::true_type{}, std::integral_constant<int, 4>{});
                 else if constexpr (!kSplit) sweep(std::true_type{}, std::integral_constant<int, 0>{});
