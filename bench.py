@@ -132,16 +132,18 @@ def kernel_source_hash() -> str:
     return h.hexdigest()[:16]
 
 
-def profiled_record(name: str):
-    """A committed ncu summary (profiles/*.json), or None when it is missing
-    or its kernel-source hash no longer matches the current sources."""
+def profiled_record(name: str, n: int):
+    """A committed ncu summary (profiles/*.json) of a system of n rows, or None
+    when it is missing, its kernel-source hash no longer matches the current
+    sources, or it was captured at another size (how much of a sweep's data the
+    L2 keeps depends on the size)."""
     path = os.path.join(ROOT, "profiles", name)
     try:
         with open(path) as f:
             d = json.load(f)
     except Exception:
         return None
-    if d.get("source_hash") != kernel_source_hash():
+    if d.get("source_hash") != kernel_source_hash() or d.get("n") != n:
         return None
     return d
 
@@ -154,6 +156,13 @@ def passes_per_iter(l: int, method: str, paired: bool = False) -> int:
     if method == "cg":
         return 10
     return 3 * (l + 1) + (2 if paired else 4) + max(0, l - 3)
+
+
+def pairs_px(l: int, prec: str, nx: int) -> bool:
+    """Whether the whole-grid stencil sweep takes two steps of p and x every
+    second iteration: 16 bytes of rows per thread (lines of whole vectors, or
+    padded ones, l <= 3), except FP64 p(1)-CG."""
+    return not (l == 1 and prec == "fp64") and (nx % (2 if prec == "fp64" else 4) == 0 or (l <= 3 and nx >= 16))
 
 
 def dp_flops_per_point(l: int) -> int:
@@ -171,20 +180,22 @@ def dp_flops_per_point(l: int) -> int:
 DP_PIPE_FLOPS_L1 = 16
 
 
-def stencil_roofline(*, n, nx, l, prec, iters, seconds, hbm_peak, hbm_src, dp_peak_tf, dp_src, rec=None):
+def stencil_roofline(*, n, nx, l, prec, iters, seconds, hbm_peak, hbm_src, dp_peak_tf, dp_src, rec=None,
+                     paired=False):
     """The roofline object of the 3D 7-point p(l)-CG solve (one launch of
     ``iters`` iterations and 2 FP64 residual sweeps in ``seconds``): the HBM
     fraction (algorithmic bytes over the measured copy bandwidth) and, for
     FP64 sweeps, the FP64 one (flops over the measured FMA rate); "bound"
     names the larger, the other sits beside it.  ``rec``: the committed ncu
-    record of the same kernel (DRAM bytes per row per sweep), or None."""
+    record of the same kernel and size (DRAM bytes per row per sweep), or None;
+    ``paired``: pairs_px of this solve."""
     vb = 8 if prec == "fp64" else 4
-    bytes_iter = passes_per_iter(l, "plcg") * vb * n
+    bytes_iter = passes_per_iter(l, "plcg", paired) * vb * n
     bytes_launch = iters * bytes_iter + 3 * 8 * n * 2   # + 2 FP64 residual sweeps
     achieved_gbs = bytes_launch / seconds / 1e9
     achieved_dp_tf = iters * dp_flops_per_point(l) * n / seconds / 1e12
     # measured DRAM traffic per launch: bytes per row per sweep of an ncu
-    # capture (smaller grid, same kernel) x rows x sweeps of this solve
+    # capture (same kernel and size, fewer iterations) x rows x sweeps of this solve
     traffic = None if rec is None else round(rec["dram_bytes_per_point_iter"] * n * (iters + 2))
     hbm_frac = achieved_gbs / hbm_peak
     dp_frac = achieved_dp_tf / dp_peak_tf
@@ -332,10 +343,11 @@ def run_ours(args):
         dp_peak_tf, dp_src = round(plcg.measure_fp64_fma_rate() / 1e12, 4), "measured (plcg_measure_fp64_fma_rate)"
     except Exception as exc:   # noqa: BLE001
         dp_peak_tf, dp_src = 1.25, f"nominal (measurement failed: {exc})"
-    rec = profiled_record("plcg_3d_fp64_l1.json") if (args.prec, args.l) == ("fp64", 1) else None
+    rec = profiled_record("plcg_3d_fp64_l1.json", n) if (args.prec, args.l) == ("fp64", 1) else None
     roofline = stencil_roofline(n=n, nx=args.nx, l=args.l, prec=args.prec, iters=statistics.mean(iters),
                                 seconds=statistics.mean(kern_s), hbm_peak=hbm_peak, hbm_src=hbm_src,
-                                dp_peak_tf=dp_peak_tf, dp_src=dp_src, rec=rec)
+                                dp_peak_tf=dp_peak_tf, dp_src=dp_src, rec=rec,
+                                paired=pairs_px(args.l, args.prec, args.nx))
     achieved_gbs = roofline["hbm"]["achieved"] if "hbm" in roofline else roofline["achieved"]
 
     extra = {}
@@ -355,7 +367,7 @@ def run_ours(args):
             r = A.solve(b, xl, l=l, interval=interval, rtol=RTOL)
             sweep[f"l{l}"] = {"iters": r.iters, "time_to_rtol_s": round(r.seconds, 5),
                               "iters_per_s": round(r.iters / r.seconds, 1),
-                              "hbm_gbs": round(r.iters * passes_per_iter(l, "plcg", l >= 2) * 8 * n
+                              "hbm_gbs": round(r.iters * passes_per_iter(l, "plcg", pairs_px(l, "fp64", args.nx)) * 8 * n
                                                / r.seconds / 1e9, 1)}
         extra["plcg_l_sweep_fp64"] = sweep
         # FP32 vectors with FP64 dots / scalars / refinement
@@ -367,8 +379,8 @@ def run_ours(args):
             r = A.solve(b, xf, l=l, interval=interval, rtol=RTOL, prec="fp32")
             xf_np = xf.cpu().numpy()
             err = float(np.linalg.norm(b_np - W.rhs(op, xf_np)) / np.linalg.norm(b_np))
-            byt = r.iters * passes_per_iter(l, "plcg", True) * 4 * n
-            rec32 = profiled_record("plcg_3d_fp32_l1.json") if l == 1 else None
+            byt = r.iters * passes_per_iter(l, "plcg", pairs_px(l, "fp32", args.nx)) * 4 * n
+            rec32 = profiled_record("plcg_3d_fp32_l1.json", n) if l == 1 else None
             mp[f"l{l}"] = {"iters": r.iters, "refinements": r.refinements,
                            "traffic": None if rec32 is None else
                            round(rec32["dram_bytes_per_point_iter"] * n * (r.iters + 2 * (r.refinements + 1))),
