@@ -67,6 +67,7 @@ extern "C" void plcg_debug_force_barrier_timeout(int on) { g_force_timeout = on;
 // and above ~2x10^4 rows the grid wins throughout.
 constexpr int64_t kClusterRowsDefault = 12288;
 constexpr int64_t kVec1Rows = 16384;
+constexpr int64_t kPadRows = 3 << 14;   // rows from which lines are padded (see build_solve)
 // p(l)-CG with l <= 2 on stencils in 16-byte row groups: whether the sweep's
 // operands are copied a unit ahead (two CTAs per SM; the others have three, or
 // FP64 p(2) two).  us per iteration without and with: FP64 3D 128^3 p(1) 48.6
@@ -75,11 +76,8 @@ constexpr int64_t kVec1Rows = 16384;
 // 128^3; FP32 p(1) 80^3 15.1 and 13.5, 112^3 17.8 and 17.6, 176^3 47.6 and 40.8,
 // but between (its vectors fit the L2, and the third CTA hides more of the
 // latency) 136 x 125 x 118 15.3 and 15.6, 128^3 20.0 and 20.4, 144^3 25.3 and 25.6.
-constexpr int64_t kPadRows = 3 << 14;   // rows from which lines are padded (see build_solve)
-
 static bool copies_ahead(bool f32, int l, int64_t n)
 {
-    // (the 2 l + 1 dots' loop does not copy ahead)
     if (!f32) return n >= (5 << 18);
     return l != 1 || n < (7 << 18) || n >= (3 << 20);
 }
@@ -570,7 +568,8 @@ static plcg_status build_solve(const plcg_matrix *A, const double *b, double *x,
                      (int64_t)pitch * A->st.ny * A->st.nz < (int64_t(1) << 31);
     const int64_t nv = pad ? (int64_t)pitch * A->st.ny * A->st.nz : n;   // rows of the solver's vectors
     if (pad) vec = want;
-    // the sweep's operands copied a unit ahead
+    // the sweep's operands copied a unit ahead (not in the 2 l + 1 dots' loop; with
+    // padded lines it is in the kernel that copies ahead, and runs without)
     const bool ahead = op == kOpStencil && !cg && l <= 2 && vec > 1 &&
                        (pad || (copies_ahead(f32, l, n) && !prm->dots_2l1));
     const void *func = pad     ? kptr_st_pad(f32, cg ? 0 : l)

@@ -1,11 +1,14 @@
 // resident.cuh -- p(l)-CG of small and mid-sized stencil systems with every
-// row's state in registers (l <= 3, R = 1, 2 or 4 rows per thread).
+// row's state in its thread (l <= 3, R = 1, 2 or 4 rows per thread).
 //
 // An iteration of a small system is a chain of latencies, not a stream of
 // bytes.  Here a thread keeps its rows for the whole solve -- z^(l)_i and
 // z^(l)_{i-1}, the current and previous vector of every other basis, phat and
 // x in registers -- and only z^(l)_{i+1} goes to global memory, for the
-// neighbours.  What bounds an iteration on GB300 then: an FP64 warp instruction
+// neighbours.  (At 512 threads a block there are 128 registers: the compiler keeps
+// part of a thread's state in local memory, in the L1 -- 270 bytes of spill stores
+// in the code for FP32, l = 1, R = 1 up to 1600 for FP64, l = 3, R = 4.)
+// What bounds an iteration on GB300 then: an FP64 warp instruction
 // takes 64 cycles on its SM sub-partition whether one lane or all are active,
 // so the scalar chain and the reductions cost as much as the sweep, and an L2
 // round trip costs about ten of them.  Hence
@@ -453,8 +456,6 @@ __device__ __forceinline__ void res_crit(ResSmem<T, L> &s, int i, T kc, T kn, co
     __syncwarp();
 }
 
-// Neighbours of a row inside the grid, bits 0 .. 5: left, right, y-, y+, z-,
-// z+; bit 6: there is no row.
 // The sum of the neighbour values x (FP64: in fixed point, fxsum.h -- 3D 40^3
 // p(1)-CG 5.04 us per iteration against 5.30 with FP64 additions, no
 // difference below; FP32: in the order of solver.cuh's sweep).
@@ -586,7 +587,8 @@ __device__ __forceinline__ int res_loop1(ResSmem<T, L> &s, const ResExch &ex, un
     }
 }
 
-// What a thread needs to know about its rows.
+// What a thread needs to know about its rows: their numbers and the neighbours
+// inside the grid, bits 0 .. 5: left, right, y-, y+, z-, z+; bit 6: there is no row.
 template <int R>
 struct ResRows {
     uint32_t g[R], nbr[R];
