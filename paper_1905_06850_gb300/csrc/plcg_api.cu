@@ -73,9 +73,10 @@ constexpr int64_t kPadRows = 3 << 14;   // rows from which lines are padded (see
 // FP64 p(2) two).  us per iteration without and with: FP64 3D 128^3 p(1) 48.6
 // and 47.0, p(2) 57.8 and 56.9, 112^3 36.0 and 35.6, 41.7 and 41.8, but 96^3 p(2)
 // 27.0 and 29.2, 80^3 20.0 and 21.5, 20.3 and 22.3; FP32 p(2) 25.9 and 20.4 at
-// 128^3; FP32 p(1) 80^3 15.1 and 13.5, 112^3 17.8 and 17.6, 176^3 47.6 and 40.8,
-// but between (its vectors fit the L2, and the third CTA hides more of the
-// latency) 136 x 125 x 118 15.3 and 15.6, 128^3 20.0 and 20.4, 144^3 25.3 and 25.6.
+// 128^3; FP32 p(1) 80^3 15.1 and 13.5, 176^3 47.6 and 40.8.  Where FP32 p(1) has
+// its vectors in the L2, 7 * 2^18 to 3 * 2^20 rows, the third CTA hides as much as
+// the copies do, and it stays with three: 136 x 125 x 118 17.0 and 16.8, 128^3 17.1
+// and 16.9, 136^3 18.6 and 19.0, 144^3 21.1 and 20.7.
 static bool copies_ahead(bool f32, int l, int64_t n)
 {
     if (!f32) return n >= (5 << 18);
