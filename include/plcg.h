@@ -340,7 +340,7 @@ plcg_status plcg_set_batched_launch(int ctas_per_sm, int rows_per_thread, int ve
  * up to max_rows unknowns, and to p(1)-CG up to max_rows / 2.  Process-wide;
  * 0 disables; the default is 12288.  A device that cannot place a cluster
  * falls back to the grid.  plcg_solve's p(l)-CG with l <= 3 on stencils (the
- * l + 1 dot products) keeps its vectors in registers instead, up to about
+ * l + 1 dot products) keeps every row's vectors in its thread instead, up to about
  * 270 thousand rows, and takes a cluster only up to a max_rows raised above the
  * default.  Errors: PLCG_ERR_INVALID (max_rows < 0). */
 plcg_status plcg_set_cluster_rows(int64_t max_rows);

@@ -6,7 +6,7 @@
 // z^(l)_{i-1}, the current and previous vector of every other basis, phat and
 // x in registers -- and only z^(l)_{i+1} goes to global memory, for the
 // neighbours.  (At 512 threads a block there are 128 registers: the compiler keeps
-// part of a thread's state in local memory, in the L1 -- 270 bytes of spill stores
+// part of a thread's state in local memory, in the L1 -- 290 bytes of spill stores
 // in the code for FP32, l = 1, R = 1 up to 1600 for FP64, l = 3, R = 4.)
 // What bounds an iteration on GB300 then: an FP64 warp instruction
 // takes 64 cycles on its SM sub-partition whether one lane or all are active,
