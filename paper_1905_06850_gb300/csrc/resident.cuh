@@ -40,18 +40,27 @@
 
 namespace plcg {
 
-// A dot's FP32 sum and its error, widened and added: by widen_f32 where both are
-// zero or normal; subnormals, infinities and NaN take the conversions (out of
-// line: inlined, they were issued ahead of the test, and a conversion costs as
-// much as any FP64 instruction -- 3D 50^3 p(1)-CG 4.7 -> 5.0 us per iteration).
+// FP32 dots (sum and error) widened and added: with widen_f32 where all are zero
+// or normal; subnormals, infinities and NaN take the conversions (out of line:
+// inlined, they were issued ahead of the test, and a conversion costs as much as
+// any FP64 instruction -- 3D 50^3 p(1)-CG 4.7 -> 5.0 us per iteration).
 static __device__ __noinline__ double widened_sum_any(float s, float t) { return (double)s + (double)t; }
 
-__device__ __forceinline__ double widened_sum(float s, float t)
+template <int N, class Acc>
+__device__ __forceinline__ void widened_sums(const Acc (&d)[N], double (&v)[N])
 {
-    const uint32_t a = __float_as_uint(s) & 0x7fffffffu, b = __float_as_uint(t) & 0x7fffffffu;
-    const bool plain = (a - 0x00800000u < 0x7f000000u || a == 0u) && (b - 0x00800000u < 0x7f000000u || b == 0u);
-    if (__builtin_expect(!plain, 0)) return widened_sum_any(s, t);
-    return widen_f32(s) + widen_f32(t);
+    uint32_t lo = 0xffffffffu, hi = 0u;   // of |x| - 1 (zero: the largest) and |x|, as integers
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+        const uint32_t a = __float_as_uint(d[q].s) & 0x7fffffffu, b = __float_as_uint(d[q].t) & 0x7fffffffu;
+        lo = min(lo, min(a - 1u, b - 1u));
+        hi = max(hi, max(a, b));
+        v[q] = widen_f32(d[q].s) + widen_f32(d[q].t);
+    }
+    if (__builtin_expect(lo < 0x007fffffu || hi >= 0x7f800000u, 0)) {
+#pragma unroll
+        for (int q = 0; q < N; ++q) v[q] = widened_sum_any(d[q].s, d[q].t);
+    }
 }
 
 template <typename T, int L>
@@ -745,10 +754,11 @@ __device__ __forceinline__ int res_loop_rows(ResSmem<T, L> &s, const ResExch &ex
             c[r] = un;
         }
         double v[L + 1];
+        if constexpr (kF32) {
+            widened_sums(dac, v);
+        } else {
 #pragma unroll
-        for (int q = 0; q <= L; ++q) {
-            if constexpr (kF32) v[q] = widened_sum(dac[q].s, dac[q].t);
-            else v[q] = dac[q].acc;
+            for (int q = 0; q <= L; ++q) v[q] = dac[q].acc;
         }
         constexpr int S = L == 1 ? 1 : 2;
         const double t = warp_reduce_scatter<L + 1>(v, lane);
